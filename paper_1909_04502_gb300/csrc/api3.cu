@@ -9,6 +9,7 @@
 
 #include "../../include/rlbm.h"
 #include "d3.h"
+#include "step3x.h"
 
 using namespace rlbm;
 
@@ -26,14 +27,13 @@ struct rlbm3_handle {
   cudaStream_t stream = nullptr;
   std::vector<double> fref;       // reference populations (FP32 storage)
   bool sym = false;               // order 2 in sign-orbit form (the steps need it)
-  // order 3 run tables in sign-orbit form for the FP64 or the FP32-storage step, or null
-  std::unique_ptr<Tables3s3<double>> ts3d;
-  std::unique_ptr<Tables3s3<float>> ts3f;
-  // order 3: tables in device memory (init, fields)
-  double* dHd = nullptr;          // Q x 30 FP64 (init)
-  double* dcd = nullptr;          // Q x 4 FP64 (fields)
+  std::unique_ptr<Tables3s3> ts3f;    // order 3, FP32 storage: run tables of the step
+  // fixed-point run tables of the order in use (the FP64 steps, the fields)
+  std::unique_ptr<Tables3x<2>> tx2;
+  std::unique_ptr<Tables3x<3>> tx3;
+  // order 3: tables of init in device memory
+  double* dHd = nullptr;          // Q x 30
   double* dfref = nullptr;        // Q
-  int* doff = nullptr;            // Q
   std::string err = "no error";
   ~rlbm3_handle() {
     for (void* b : buf) cudaFree(b);
@@ -41,9 +41,7 @@ struct rlbm3_handle {
     cudaFree(staging);
     cudaFree(status);
     cudaFree(dHd);
-    cudaFree(dcd);
     cudaFree(dfref);
-    cudaFree(doff);
   }
 };
 
@@ -82,11 +80,10 @@ int upload(void** dst, const std::vector<T>& v) {
 // The order-3 run tables (sign-orbit form): 33 runs of 8 and 6 runs of 4
 // with the non-zero components x y, x z, x y, x z, y z, y z; null when the
 // table has another layout.
-template <typename S>
-std::unique_ptr<Tables3s3<S>> order3_runs(const Quadrature3& q, const std::vector<int>& offs) {
+std::unique_ptr<Tables3s3> order3_runs(const Quadrature3& q, const std::vector<int>& offs) {
   static const int kMask4[kRuns4o3] = {3, 5, 3, 5, 6, 6};
-  std::unique_ptr<Tables3s3<S>> t(new Tables3s3<S>());
-  std::memset(t.get(), 0, sizeof(Tables3s3<S>));
+  std::unique_ptr<Tables3s3> t(new Tables3s3());
+  std::memset(t.get(), 0, sizeof(Tables3s3));
   int n8 = 0, n4 = 0, i0 = 0;
   for (int mask : q.orbit_mask) {
     const int size = mask == 7 ? 8 : 4;
@@ -95,7 +92,7 @@ std::unique_ptr<Tables3s3<S>> order3_runs(const Quadrature3& q, const std::vecto
     const double mono[14] = {p[0], p[1], p[2], p[3], p[0] * p[0], p[0] * p[1], p[0] * p[2],
                              p[0] * p[3], p[1] * p[1], p[1] * p[2], p[1] * p[3], p[2] * p[2],
                              p[2] * p[3], p[3] * p[3]};
-    S *H, *mo, *v;
+    float *H, *mo, *v;
     if (mask == 7 && n8 < kRuns8o3) {
       t->start8[n8] = i0;
       H = t->H8[n8], mo = t->mono8[n8], v = t->v8[n8];
@@ -107,13 +104,12 @@ std::unique_ptr<Tables3s3<S>> order3_runs(const Quadrature3& q, const std::vecto
     } else {
       return nullptr;
     }
-    for (int k = 0; k < 30; ++k) H[k] = (S)q.H[(size_t)i0 * 30 + k];
-    for (int k = 0; k < 14; ++k) mo[k] = (S)mono[k];
-    for (int k = 0; k < 3; ++k) v[k] = (S)(p[1 + k] / p[0]);
+    for (int k = 0; k < 30; ++k) H[k] = (float)q.H[(size_t)i0 * 30 + k];
+    for (int k = 0; k < 14; ++k) mo[k] = (float)mono[k];
+    for (int k = 0; k < 3; ++k) v[k] = (float)(p[1 + k] / p[0]);
     i0 += size;
   }
   if (n8 != kRuns8o3 || n4 != kRuns4o3 || i0 != q.Q || (int)offs.size() != q.Q) return nullptr;
-  for (int i = 0; i < q.Q; ++i) t->off[i] = offs[i];
   for (int r = 0; r < kRuns8o3; ++r)
     for (int k = 0; k < 8; ++k) t->off8[r][k] = offs[t->start8[r] + k];
   for (int r = 0; r < kRuns4o3; ++r)
@@ -168,6 +164,7 @@ int rlbm3_create(int nx, int ny, int nz, double tau, int order, int precision, v
   s.slab = (long long)(ny + 2 * s.h) * s.pitch;
   s.plane = ((long long)(nz + 2 * s.h) * s.slab + 31) / 32 * 32;
   s.tau = tau;
+  s.inv_tau = 1.0 / tau;
   h->elem = precision == RLBM_FP32_STORE ? 4 : 8;
   s.n_ref = h->elem == 4 ? 1.0 : 0.0;
   s.T_ref = h->elem == 4 ? 1.0 : 0.0;
@@ -194,18 +191,26 @@ int rlbm3_create(int nx, int ny, int nz, double tau, int order, int precision, v
   h->tb.reset(new Tables3());
   std::memset(h->tb.get(), 0, sizeof(Tables3));
   if (order == 3) {
-    std::vector<double> c(4 * s.Q);
-    for (int i = 0; i < s.Q; ++i)
-      for (int u = 0; u < 4; ++u) c[4 * i + u] = h->q.p[4 * i + u];
     int rc = RLBM_OK;           // (the steps take their run tables as kernel parameters)
     if (!rc) rc = upload((void**)&h->dHd, h->q.H);
-    if (!rc) rc = upload((void**)&h->dcd, c);
     if (!rc) rc = upload((void**)&h->dfref, h->fref);
-    if (!rc) rc = upload((void**)&h->doff, offs);
     if (rc) return fail3(nullptr, rc, "order-3 tables");
   }
-  if (order == 3 && h->q.sym && h->elem == 8) h->ts3d = order3_runs<double>(h->q, offs);
-  if (order == 3 && h->q.sym && h->elem == 4) h->ts3f = order3_runs<float>(h->q, offs);
+  if (order == 3 && h->q.sym && h->elem == 4) h->ts3f = order3_runs(h->q, offs);
+  {
+    std::vector<int> shift(s.Q);
+    for (int i = 0; i < s.Q; ++i)
+      shift[i] = (int)((long long)offs[i] - (order == 2 ? (long long)i * s.plane : 0));
+    bool ok;
+    if (order == 2) {
+      h->tx2.reset(new Tables3x<2>());
+      ok = fill_tables3x<2>(h->q, shift.data(), h->fref.data(), h->tx2.get());
+    } else {
+      h->tx3.reset(new Tables3x<3>());
+      ok = fill_tables3x<3>(h->q, shift.data(), h->fref.data(), h->tx3.get());
+    }
+    if (!ok) return fail3(nullptr, RLBM_ERR_QUADRATURE, "3-d table not in sign-orbit form");
+  }
   if (order == 2) {
     // sign-orbit form: 9 runs of 8, then the axis pairs along x, y and z
     static const int kMasks[kRuns3] = {7, 7, 7, 7, 7, 7, 7, 7, 7, 1, 2, 4};
@@ -216,18 +221,15 @@ int rlbm3_create(int nx, int ny, int nz, double tau, int order, int precision, v
       const double mono[14] = {p[0], p[1], p[2], p[3], p[0] * p[0], p[0] * p[1], p[0] * p[2],
                                p[0] * p[3], p[1] * p[1], p[1] * p[2], p[1] * p[3], p[2] * p[2],
                                p[2] * p[3], p[3] * p[3]};
-      for (int k = 0; k < 14; ++k) h->tb->mono[r][k] = mono[k];
       for (int k = 0; k < 14; ++k) h->tb->monof[r][k] = (float)mono[k];
     }
   }
   // the steps take the table in sign-orbit form (checked exactly above)
-  if (order == 2 ? !h->sym : !(h->elem == 8 ? (bool)h->ts3d : (bool)h->ts3f))
+  if (order == 2 ? !h->sym : (h->elem == 4 && !h->ts3f))
     return fail3(nullptr, RLBM_ERR_QUADRATURE, "3-d table not in sign-orbit form");
   for (int i = 0; i < s.Q && order == 2; ++i) {
-    for (int u = 0; u < 4; ++u) h->tb->c[i][u] = h->q.p[4 * i + u];
-    for (int u = 0; u < 3; ++u) h->tb->v[i][u] = h->q.p[4 * i + 1 + u] / h->q.p[4 * i];
     for (int k = 0; k < 14; ++k) h->tb->H[i][k] = h->q.H[(size_t)i * 14 + k];
-    for (int u = 0; u < 3; ++u) h->tb->vf[i][u] = (float)h->tb->v[i][u];
+    for (int u = 0; u < 3; ++u) h->tb->vf[i][u] = (float)(h->q.p[4 * i + 1 + u] / h->q.p[4 * i]);
     for (int k = 0; k < 14; ++k) h->tb->Hf[i][k] = (float)h->tb->H[i][k];
     h->tb->fref[i] = h->fref[i];
     h->tb->off[i] = offs[i];
@@ -314,20 +316,15 @@ int rlbm3_step(rlbm3_handle* h, int nsteps) {
   if (!h || nsteps < 0) return fail3(h, RLBM_ERR_INVALID_ARG, "bad argument");
   for (int t = 0; t < nsteps; ++t) {
     cudaError_t e;
-    if (h->q.order == 3) {
-      if (h->elem == 4) {
-        Step3qArgs<float> a{(const float*)h->buf[h->cur], (float*)h->buf[h->cur ^ 1], h->status, h->sc};
-        e = launch_step3q_symf(*h->ts3f, a, h->stream);
-      } else {
-        Step3qArgs<double> a{(const double*)h->buf[h->cur], (double*)h->buf[h->cur ^ 1], h->status, h->sc};
-        e = launch_step3q_sym(*h->ts3d, a, h->stream);
-      }
-    } else if (h->elem == 4) {
+    if (h->elem == 8) {
+      Step3Args<double> a{(const double*)h->buf[h->cur], (double*)h->buf[h->cur ^ 1], h->status, h->sc};
+      e = h->q.order == 3 ? launch_step3x<3>(*h->tx3, a, h->stream) : launch_step3x<2>(*h->tx2, a, h->stream);
+    } else if (h->q.order == 3) {
+      Step3qArgs<float> a{(const float*)h->buf[h->cur], (float*)h->buf[h->cur ^ 1], h->status, h->sc};
+      e = launch_step3q_symf(*h->ts3f, a, h->stream);
+    } else {
       Step3Args<float> a{(const float*)h->buf[h->cur], (float*)h->buf[h->cur ^ 1], h->status, h->sc};
       e = launch_step3f_sym(*h->tb, a, h->stream);
-    } else {
-      Step3Args<double> a{(const double*)h->buf[h->cur], (double*)h->buf[h->cur ^ 1], h->status, h->sc};
-      e = launch_step3_sym(*h->tb, a, h->stream);
     }
     if (e != cudaSuccess) return cuda_fail3(h, e, "step kernel");
     h->cur ^= 1;
@@ -343,20 +340,12 @@ int rlbm3_moments(rlbm3_handle* h, double* out, int on_device) {
   double* dst = on_device ? out : h->fields;
   const int pull = h->have_prev ? 1 : 0;
   cudaError_t e;
-  if (h->q.order == 3) {
-    if (h->elem == 4) {
-      Fields3qArgs<float> a{(const float*)fin, pull, dst, h->sc, h->dcd, h->doff, h->dfref};
-      e = launch_fields3q<float>(a, h->stream);
-    } else {
-      Fields3qArgs<double> a{(const double*)fin, pull, dst, h->sc, h->dcd, h->doff, h->dfref};
-      e = launch_fields3q<double>(a, h->stream);
-    }
-  } else if (h->elem == 4) {
+  if (h->elem == 4) {
     Fields3Args<float> a{(const float*)fin, pull, dst, h->sc};
-    e = launch_fields3<float>(*h->tb, a, h->stream);
+    e = h->q.order == 3 ? launch_fields3x<3, float>(*h->tx3, a, h->stream) : launch_fields3x<2, float>(*h->tx2, a, h->stream);
   } else {
     Fields3Args<double> a{(const double*)fin, pull, dst, h->sc};
-    e = launch_fields3<double>(*h->tb, a, h->stream);
+    e = h->q.order == 3 ? launch_fields3x<3, double>(*h->tx3, a, h->stream) : launch_fields3x<2, double>(*h->tx2, a, h->stream);
   }
   if (e != cudaSuccess) return cuda_fail3(h, e, "fields kernel");
   if (!on_device) {

@@ -76,55 +76,6 @@ __device__ __forceinline__ void dadj_col0(const R (&B)[4][4], R (&d)[4]) {
   d[3] = -((B[2][0] * B[3][2] - B[2][2] * B[3][0]) + (B[1][0] * B[3][1] - B[1][1] * B[3][0]));
 }
 
-struct Macro3 {
-  double n, T, eps, U[4];
-  bool ok;
-};
-
-// Largest eigenvalue eps of A^a_b = T^ac eta_cb and its timelike eigenvector:
-// Newton on p(l) = det(A - l I) from the ideal-fluid root for P = eps / 3,
-// p'(l) = -(sum of the principal 3 x 3 minors of A - l I); U from the first
-// column of adj(A - l I) (a right null vector), normalised to U.U = 1, U^0 > 0.
-__device__ __forceinline__ Macro3 landau3(const double (&N)[4], const double (&Tm)[4][4]) {
-  double A[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) A[a][b] = b == 0 ? Tm[a][b] : -Tm[a][b];
-  const double E = Tm[0][0], M2 = Tm[0][1] * Tm[0][1] + Tm[0][2] * Tm[0][2] + Tm[0][3] * Tm[0][3];
-  const double k = 1.0 / 3.0;
-  double lam = (-(1.0 - k) * E + sqrt(fmax((1.0 - k) * (1.0 - k) * E * E + 4.0 * k * (E * E - M2), 0.0))) /
-               (2.0 * k);
-  double B[4][4];
-  for (int it = 0; it < 8; ++it) {
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) B[a][b] = A[a][b] - (a == b ? lam : 0.0);
-    const double dp = ddet4(B);
-    if (!(dp != 0.0)) break;
-    const double step = det4(B) / dp;
-    lam -= step;
-    if (fabs(step) <= 1e-15 * fabs(lam)) break;
-  }
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) B[a][b] = A[a][b] - (a == b ? lam : 0.0);
-  double v[4];
-  adj_col0(B, v);
-  const double nu2 = v[0] * v[0] - v[1] * v[1] - v[2] * v[2] - v[3] * v[3];
-  Macro3 M;
-  const double inu = (v[0] > 0.0 ? 1.0 : -1.0) / sqrt(fabs(nu2));
-#pragma unroll
-  for (int a = 0; a < 4; ++a) M.U[a] = v[a] * inu;
-  M.n = M.U[0] * N[0] - M.U[1] * N[1] - M.U[2] * N[2] - M.U[3] * N[3];
-  M.eps = lam;
-  M.T = lam / (3.0 * M.n);
-  M.ok = nu2 > 0.0 && M.n > 0.0 && M.T > 0.0 && isfinite(M.T) && isfinite(M.U[0]);
-  return M;
-}
-
 // MJ moments of the basis 1 | p0 px py pz | p0px p0py p0pz pxpx pxpy pxpz pypy
 // pypz pzpz for massless particles in d = 3 (App. B): <1> = n/(2T),
 // <p^a> = n U^a, <p^a p^b> = n (4T U^a U^b - T eta^ab).
@@ -318,22 +269,14 @@ __device__ __forceinline__ void mj_delta3(const Macro3f& M, float nr, float Tr, 
   }
 }
 
-// The collision frame from the 14 moment sums m = N0 Nx Ny Nz T00 T0x T0y
-// T0z Txx Txy Txz Tyy Tyz Tzz (of f in FP64 storage, of g = f - f_ref in FP32
-// storage): the moments Mk of the K-member basis that the equilibrium H Mk
-// needs (full moments in FP64, differences from the reference in FP32), and
+// The collision frame of FP32 storage from the 14 moment sums m = N0 Nx Ny Nz
+// T00 T0x T0y T0z Txx Txy Txz Tyy Tyz Tzz of g = f - f_ref: the moments Mk of
+// the K-member basis, as differences from the reference, and
 // tau^-1 U (zero where the cell has no Landau frame, which leaves it
 // unrelaxed).  Returns whether the frame exists.
 // A cell without a physical Landau frame is left unrelaxed (Omega = 0); its
 // frame is replaced by the reference state (rest, n_ref or 1, T_ref) so
 // that the equilibrium and Omega stay finite (0 * NaN is not 0).
-__device__ __forceinline__ void unphysical_to_reference3(const Scalars3& s, Macro3& M) {
-  M.n = s.n_ref > 0.0 ? s.n_ref : 1.0;
-  M.T = s.T_ref;
-  M.eps = 3.0 * M.n * M.T;
-  M.U[0] = 1.0;
-  M.U[1] = M.U[2] = M.U[3] = 0.0;
-}
 __device__ __forceinline__ void unphysical_to_reference3(const Scalars3& s, Macro3f& M) {
   M.n = (float)(s.n_ref > 0.0 ? s.n_ref : 1.0);
   M.T = s.f_T_ref;
@@ -342,39 +285,23 @@ __device__ __forceinline__ void unphysical_to_reference3(const Scalars3& s, Macr
   M.Ux = M.Uy = M.Uz = 0.f;
 }
 
-template <typename S, int K>
-__device__ __forceinline__ bool frame3(const S (&m)[14], const Scalars3& s, S (&Mk)[K], S& kU0, S (&kU)[3]) {
-  if constexpr (sizeof(S) == 8) {
-    const double N[4] = {m[0], m[1], m[2], m[3]};
-    const double Tm[4][4] = {{m[4], m[5], m[6], m[7]},
-                             {m[5], m[8], m[9], m[10]},
-                             {m[6], m[9], m[11], m[12]},
-                             {m[7], m[10], m[12], m[13]}};
-    Macro3 M = landau3(N, Tm);
-    if (!M.ok) unphysical_to_reference3(s, M);
-    mj_full3<K>(M.n, M.T, M.U, Mk);
-    const double kt = M.ok ? 1.0 / s.tau : 0.0;
-    kU0 = kt * M.U[0];
-    kU[0] = kt * M.U[1];
-    kU[1] = kt * M.U[2];
-    kU[2] = kt * M.U[3];
-    return M.ok;
-  } else {
-    const float N[4] = {m[0], m[1], m[2], m[3]};
-    const float Tm[4][4] = {{m[4], m[5], m[6], m[7]},
-                            {m[5], m[8], m[9], m[10]},
-                            {m[6], m[9], m[11], m[12]},
-                            {m[7], m[10], m[12], m[13]}};
-    Macro3f M = landau3f(N, Tm, s);
-    if (!M.ok) unphysical_to_reference3(s, M);
-    mj_delta3<K>(M, s.f_n_ref, s.f_T_ref, Mk);
-    const float kt = M.ok ? s.f_inv_tau : 0.f;
-    kU0 = kt * M.U0;
-    kU[0] = kt * M.Ux;
-    kU[1] = kt * M.Uy;
-    kU[2] = kt * M.Uz;
-    return M.ok;
-  }
+template <int K>
+__device__ __forceinline__ bool frame3(const float (&m)[14], const Scalars3& s, float (&Mk)[K], float& kU0,
+                                       float (&kU)[3]) {
+  const float N[4] = {m[0], m[1], m[2], m[3]};
+  const float Tm[4][4] = {{m[4], m[5], m[6], m[7]},
+                          {m[5], m[8], m[9], m[10]},
+                          {m[6], m[9], m[11], m[12]},
+                          {m[7], m[10], m[12], m[13]}};
+  Macro3f M = landau3f(N, Tm, s);
+  if (!M.ok) unphysical_to_reference3(s, M);
+  mj_delta3<K>(M, s.f_n_ref, s.f_T_ref, Mk);
+  const float kt = M.ok ? s.f_inv_tau : 0.f;
+  kU0 = kt * M.U0;
+  kU[0] = kt * M.Ux;
+  kU[1] = kt * M.Uy;
+  kU[2] = kt * M.Uz;
+  return M.ok;
 }
 
 // Walsh-Hadamard transform in place: v[c] <- sum_s (-1)^{popcount(c & s)} v[s]
@@ -411,12 +338,12 @@ __device__ __forceinline__ void moments_run8(const S (&F)[8], const C* c, S (&m)
   m[13] = fma((S)c[13], F[0], m[13]);
 }
 
-// FP32 storage: the periodic images of a cell next to a face, copied from the
+// The periodic images of a cell next to a face, copied from the
 // values the thread has just stored for the cell itself, B populations at a
 // time so that B loads are in flight (one at a time, each waits on the L2
 // round trip of the one before, as the stores in between may alias them).
-template <int QT, int B>
-__device__ __forceinline__ void images_from_stored(const Scalars3& s, float* out, long long si, int x, int y, int z) {
+template <int QT, int B, typename S>
+__device__ __forceinline__ void images_from_stored(const Scalars3& s, S* out, long long si, int x, int y, int z) {
   int ix[2], iy[2], iz[2];
   const int nx2 = images1(x, s.nx, s.h, ix), ny2 = images1(y, s.ny, s.h, iy), nz2 = images1(z, s.nz, s.h, iz);
   if (nx2 + ny2 + nz2 == 0) return;
@@ -431,12 +358,12 @@ __device__ __forceinline__ void images_from_stored(const Scalars3& s, float* out
   static_assert(QT % B == 0, "whole batches");
   const long long P = s.plane;
   for (int i0 = 0; i0 < QT; i0 += B) {
-    float v[B];
+    S v[B];
 #pragma unroll
     for (int j = 0; j < B; ++j) v[j] = out[(long long)(i0 + j) * P + si];
 #pragma unroll
     for (int j = 0; j < B; ++j) {
-      float* oi = out + (long long)(i0 + j) * P;
+      S* oi = out + (long long)(i0 + j) * P;
       for (int m = 0; m < nimg; ++m) oi[img[m]] = v[j];
     }
   }
