@@ -585,7 +585,7 @@ cudaError_t fwd_step(rlbm_handle* h, const void* src, void* dst, float* macro, c
     return launch_step<float>(*h->tf, a, mode, st);
   }
   StepArgs<double> a{h->sc, (const double*)src, (double*)dst, (const double*)h->tau_field, h->status};
-  return launch_step<double>(*h->td, a, mode, st);
+  return h->tx ? launch_step2x(*h->tx, a, mode, st) : launch_step<double>(*h->td, a, mode, st);
 }
 
 void free_adjoint(rlbm_adjoint* A) {

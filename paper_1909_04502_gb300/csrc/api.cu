@@ -11,6 +11,7 @@
 #include "../../include/rlbm.h"
 #include "dispatch.h"
 #include "handle.h"
+#include "step2x.h"
 #include "step_impl.cuh"
 #include "setup.h"
 
@@ -92,6 +93,7 @@ void finish_scalars(Scalars* s) {
   s->f_wall_T[1] = (float)s->wall_T[1];
   s->massless = (s->m == 0.0) ? 1 : 0;
   s->iplane = (int)s->plane;
+  s->inv_tau = 1.0 / s->tau;
   s->f_tau = (float)s->tau;
   s->f_tau_coef = (float)s->tau_coef;
   s->f_m = (float)s->m;
@@ -503,6 +505,10 @@ int rlbm_create(const rlbm_params* p, rlbm_handle** out) {
   } else {
     h->td.reset(new Tables<double>());
     fill_tables(h.get(), s, h->td.get());
+    if (s.sym) {
+      h->tx.reset(new Tables2x());
+      if (!fill_tables2x(h->q, h->H, h->K, s, *h->td, h->tx.get())) h->tx.reset();
+    }
   }
   // device buffers
   const size_t pop_bytes = (size_t)h->q.Q * s.plane * h->elem;
@@ -650,7 +656,7 @@ int rlbm_step(rlbm_handle* h, int nsteps) {
     } else {
       StepArgs<double> a{h->sc, (const double*)h->buf[h->cur], (double*)h->buf[h->cur ^ 1],
                          (const double*)h->tau_field, h->status};
-      e = launch_step<double>(*h->td, a, mode, h->stream);
+      e = h->tx ? launch_step2x(*h->tx, a, mode, h->stream) : launch_step<double>(*h->td, a, mode, h->stream);
     }
     if (e != cudaSuccess) return cuda_fail(h, e, "step kernel");
     h->cur ^= 1;
@@ -665,27 +671,35 @@ int rlbm_moments(rlbm_handle* h, double* n, double* ux, double* uy, double* T, d
   if (!h) return RLBM_ERR_INVALID_ARG;
   const Scalars& s = h->sc;
   const int mode = h->p.stream_mode == RLBM_BILINEAR ? kBilinear : kOnLattice;
-  const int want = (Nab || Tab) ? 1 : 0;
   const void* fin = h->have_prev ? h->buf[h->cur ^ 1] : h->buf[h->cur];
+  // device outputs are written by the kernel itself; host outputs go through the field planes
+  double* host[7] = {n, ux, uy, T, eps, Nab, Tab};
+  double* dev[7];
+  for (int k = 0; k < 7; ++k)
+    dev[k] = !host[k] || on_device ? host[k] : h->fields + (size_t)(k == 6 ? 8 : k) * s.ncell;
+  auto fill = [&](auto& a) {
+    for (int k = 0; k < 5; ++k) a.out[k] = dev[k];
+    a.N = dev[5];
+    a.Tab = dev[6];
+    a.status = h->status;
+  };
   cudaError_t e;
   if (h->elem == 4) {
-    MomentArgs<float> a{s, (const float*)fin, h->have_prev ? 1 : 0, h->fields, want, h->status};
+    MomentArgs<float> a{s, (const float*)fin, h->have_prev ? 1 : 0};
+    fill(a);
     e = launch_fields<float>(*h->tf, a, mode, h->stream);
   } else {
-    MomentArgs<double> a{s, (const double*)fin, h->have_prev ? 1 : 0, h->fields, want, h->status};
-    e = launch_fields<double>(*h->td, a, mode, h->stream);
+    MomentArgs<double> a{s, (const double*)fin, h->have_prev ? 1 : 0};
+    fill(a);
+    e = h->tx ? launch_fields2x(*h->tx, a, mode, h->stream) : launch_fields<double>(*h->td, a, mode, h->stream);
   }
   if (e != cudaSuccess) return cuda_fail(h, e, "fields kernel");
-  const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-  const size_t bytes = (size_t)s.ncell * sizeof(double);
-  double* outs[5] = {n, ux, uy, T, eps};
-  for (int k = 0; k < 5; ++k)
-    if (outs[k]) RLBM_CUDA(h, cudaMemcpyAsync(outs[k], h->fields + (size_t)k * s.ncell, bytes, kind, h->stream));
-  for (int k = 0; k < 3; ++k)
-    if (Nab) RLBM_CUDA(h, cudaMemcpyAsync(Nab + (size_t)k * s.ncell, h->fields + (size_t)(5 + k) * s.ncell, bytes, kind, h->stream));
-  for (int k = 0; k < 6; ++k)
-    if (Tab) RLBM_CUDA(h, cudaMemcpyAsync(Tab + (size_t)k * s.ncell, h->fields + (size_t)(8 + k) * s.ncell, bytes, kind, h->stream));
-  if (!on_device) RLBM_CUDA(h, cudaStreamSynchronize(h->stream));
+  if (on_device) return RLBM_OK;
+  for (int k = 0; k < 7; ++k) {
+    const size_t bytes = (size_t)(k < 5 ? 1 : k == 5 ? 3 : 6) * s.ncell * sizeof(double);
+    if (host[k]) RLBM_CUDA(h, cudaMemcpyAsync(host[k], dev[k], bytes, cudaMemcpyDeviceToHost, h->stream));
+  }
+  RLBM_CUDA(h, cudaStreamSynchronize(h->stream));
   return RLBM_OK;
 }
 
@@ -773,7 +787,7 @@ int rlbm_buffers(rlbm_handle* h, void** cur, void** prev, int* elem_size, long l
 void rlbm_internal_set_error(const std::string& msg) { g_create_error = msg; }
 
 int rlbm_internal_prepare(const rlbm_params* p, Scalars* sc, Tables<float>* tf, Tables<double>* td,
-                          std::unique_ptr<XeqTables>* txq, std::string* err) {
+                          std::unique_ptr<XeqTables>* txq, std::unique_ptr<Tables2x>* tx, std::string* err) {
   {
     const int vrc = validate_params(p, err);
     if (vrc != RLBM_OK) return vrc;
@@ -834,6 +848,10 @@ int rlbm_internal_prepare(const rlbm_params* p, Scalars* sc, Tables<float>* tf, 
     }
   } else {
     fill_tables(&h, s, td);
+    if (s.sym) {
+      tx->reset(new Tables2x());
+      if (!fill_tables2x(h.q, h.H, h.K, s, *td, tx->get())) tx->reset();
+    }
   }
   return RLBM_OK;
 }

@@ -8,7 +8,7 @@
 // run on the integer pipes, and only the macroscopic state of the cell, some
 // hundred operations, stays in FP64.
 //
-// Precision.  Moments: X_i = f_i 2^(e_i) in units of 2^(E - 59), e_i a constant
+// Precision.  Moments: X_i = f_i 2^(e_i) in units of 2^(E - 59) or 2^(E - 60), e_i a constant
 // of the table (the exponent of p0^2, so that 2^-59 is relative to the largest
 // contribution to T^00) and 2^E above them all.  Relaxation: f and f^eq of a
 // run in units of 2^(u - 58), 2^u above the run's own populations and, with
@@ -25,7 +25,8 @@
 namespace rlbm {
 
 constexpr int kBits = 58;        // populations in a relaxation: |X| < 2^kBits
-constexpr int kBitsM = 59;       // populations in the moment sums
+constexpr int kBitsM = 59;       // populations in the moment sums: runs of 8 members
+constexpr int kBitsM4 = 60;      // ... and of at most 4
 constexpr int kHead = 4;         // results of a relaxation: below 2^(kBits + kHead)
 constexpr int kCoefM = 63;       // moment constants: their sum over the runs at most 2^kCoefM
 constexpr int kCoefH = 60;       // equilibrium constants: a row's sum over a parity class at most four
@@ -122,10 +123,11 @@ __host__ __device__ __forceinline__ long long to_fixed_positive(double f, int d)
   const unsigned long long m = (bits_of(f) & 0x000FFFFFFFFFFFFFULL) | 0x0010000000000000ULL;
   return (long long)((shift_right(m << (kBits - 52), d) + 1) >> 1);
 }
-// |f| in units of 2^(u - kBitsM), the bits below the unit cut
+// |f| in units of 2^(u - BITS), the bits below the unit cut
+template <int BITS>
 __host__ __device__ __forceinline__ long long to_fixed_cut(double f, int d) {
   const unsigned long long m = (bits_of(f) & 0x000FFFFFFFFFFFFFULL) | 0x0010000000000000ULL;
-  return (long long)shift_right(m << (kBitsM - 53), d);
+  return (long long)shift_right(m << (BITS - 53), d);
 }
 
 // The double nearest to Y 2^(k - 1023), |Y| < 2^62, k + 62 < 2047 and k > 0.

@@ -10,6 +10,7 @@
 #include "dispatch.h"
 #include "kernels.cuh"
 #include "setup.h"
+#include "step2x.h"
 #include "step_tma.h"
 
 struct rlbm_handle {
@@ -21,6 +22,7 @@ struct rlbm_handle {
   rlbm::Scalars sc;              // kernel scalars
   std::unique_ptr<rlbm::Tables<float>> tf;    // kernel tables, FP32 storage
   std::unique_ptr<rlbm::Tables<double>> td;   // kernel tables, FP64
+  std::unique_ptr<rlbm::Tables2x> tx;         // FP64, orbit-symmetric: fixed-point step (step2x.cu), else null
   std::unique_ptr<rlbm::XeqTables> txq;       // FP32 storage at order 3, m~ >= 6: extended-precision
                                               // equilibrium tables (step_xeq.cu), else null
   size_t elem = 4;               // bytes per stored population

@@ -50,7 +50,7 @@ struct Scalars {
   long long plane;
   int boundary;            // 0 periodic, 1 free-flow in x
   int tau_mode;            // 0 const, 1 field, 2 eta/s
-  double tau;              // const tau
+  double tau, inv_tau;     // const tau and its reciprocal
   double tau_coef;         // (eta/s)(d+2) kappa  (tau = tau_coef / T)
   double m;                // rest mass m~
   double n_ref, T_ref;     // reference state (n_ref = 0: no shift)
@@ -112,8 +112,9 @@ struct MomentArgs {
   Scalars s;
   const S* fin;
   int gather;            // 1: stream first (fields of S f*), 0: fields of fin itself
-  double* out;           // [14][ncell] (row-major cells): n ux uy T eps N0 Nx Ny T00 T0x T0y Txx Txy Tyy
-  int want_moments;      // write planes 5..13
+  double* out[5];        // n ux uy T eps, row-major cells (each may be null)
+  double* N;             // N0 Nx Ny planes of ncell, or null
+  double* Tab;           // T00 T0x T0y Txx Txy Tyy planes, or null
   unsigned long long* status;
 };
 

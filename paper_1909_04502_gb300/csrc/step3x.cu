@@ -27,6 +27,7 @@
 #include <cuda_runtime.h>
 
 #include "d3_impl.cuh"
+#include "fxstep.cuh"
 #include "step3x.h"
 
 namespace rlbm {
@@ -64,61 +65,17 @@ __device__ constexpr int gather_bits(int mask, int par) {
   return out;
 }
 
-template <int N>
-struct Int {
-  static constexpr int value = N;
-};
-
-// exponent x with |v| < 2^x
-__device__ __forceinline__ int above(float v) { return (int)((__float_as_uint(v) >> 23) & 0xFF) - 126; }
-
-// Raises the scale 2^E of the moment sums to hold populations below 2^want (a bit to spare).
-__device__ __forceinline__ void raise_scale(long long (&m)[kMom3], int& E, int want) {
-  if (want <= E) return;
-  const int to = want + 1, sh = min(to - E, 63);
-#pragma unroll
-  for (int k = 0; k < kMom3; ++k) m[k] >>= sh;
-  E = to;
-}
-
-// m + c X / 2^64, rounded
-__device__ __forceinline__ void add_product(long long& m, Cx c, int xh, int xl) {
-  Acc a{m, 0x80000000LL};
-  macs(a, c, xh, xl);
-  m = a.H + (long long)hi32(a.M);
-}
-
-// The largest biased exponent of a run, and whether every member is finite and not negative.
-template <int L>
-__device__ __forceinline__ int run_exponent(const double (&f)[L], bool& plain) {
-  unsigned h = 0;
-#pragma unroll
-  for (int q = 0; q < L; ++q) h = max(h, (unsigned)__double2hiint(f[q]));
-  plain = h < 0x7FF00000U;
-  if (__builtin_expect(!plain, 0)) {
-    h = 0;
-#pragma unroll
-    for (int q = 0; q < L; ++q) h = max(h, (unsigned)__double2hiint(f[q]) & 0x7FF00000U);
-  }
-  return (int)(h >> 20);
-}
-
-// Signed, subnormal and non-finite values: out of line, so that the loops of
-// the usual case stay short.
-__device__ __noinline__ long long to_fixed_any(double f, int d) { return to_fixed(f, d - biased_exponent(f)); }
-__device__ __noinline__ double from_fixed_any(long long Y, int k) { return from_fixed(Y, k); }
-
 // A run's populations scaled by 2^ep in units of 2^(E - kBitsM), E raised where
 // they need it.
 template <int L>
 __device__ __forceinline__ void run_units(const double (&f)[L], int ep, long long, long long (&m)[kMom3], int& E,
                                           long long (&X)[L]) {
   bool plain;
-  raise_scale(m, E, run_exponent(f, plain) + ep + 1);
+  raise_scale<1>(m, E, run_exponent(f, plain) + ep + 1);
   const int d = E - 1 - ep;
   if (__builtin_expect(plain, 1)) {
 #pragma unroll
-    for (int q = 0; q < L; ++q) X[q] = to_fixed_cut(f[q], d - (__double2hiint(f[q]) >> 20));
+    for (int q = 0; q < L; ++q) X[q] = to_fixed_cut<kBitsM>(f[q], d - (__double2hiint(f[q]) >> 20));
   } else {
 #pragma unroll
     for (int q = 0; q < L; ++q) X[q] = to_fixed_any(f[q], d) << (kBitsM - kBits);
@@ -132,7 +89,7 @@ __device__ __forceinline__ void run_units(const float (&g)[L], int ep, long long
   unsigned h = 0;
 #pragma unroll
   for (int q = 0; q < L; ++q) h = max(h, __float_as_uint(g[q]) & 0x7FFFFFFFU);
-  raise_scale(m, E, (int)(h >> 23) + 896 + ep + 1);
+  raise_scale<1>(m, E, (int)(h >> 23) + 896 + ep + 1);
   const int d = E - 1 - ep - 896 + 63 - kBitsM;
   const long long r = ref >> min(E - ref_E, 63);
 #pragma unroll
@@ -336,18 +293,6 @@ __device__ __forceinline__ void mj_moments3x(const Cell3& c, const double (&U)[3
     M[29] = fma(zz, U[2], 3.0 * rU[2]);
   }
 }
-
-// Values of a thread split for products (split_balanced), in a shared-memory
-// column of its own: in registers they would hold 28 to 76 of them.
-struct Column {
-  int2* s;          // [][128]
-  __device__ __forceinline__ void set(int k, long long v) const {
-    int2 x;
-    split_balanced(v, x.x, x.y);
-    s[k * 128] = x;
-  }
-  __device__ __forceinline__ int2 get(int k) const { return s[k * 128]; }
-};
 
 template <int ORDER>
 __global__ void __launch_bounds__(128, ORDER == 2 ? 6 : 5) k_step3x(const __grid_constant__ Tables3x<ORDER> tb,

@@ -4,6 +4,7 @@
 // step_o3.cu.
 #pragma once
 #include "fpconv.cuh"
+#include "fx64.cuh"
 #include "kernels.cuh"
 
 namespace rlbm {
@@ -855,8 +856,8 @@ __global__ void __launch_bounds__(kThreads, step_threads_per_sm<S, QT, MODE, SYM
   }
 }
 
-// Fields of f(t) (steps 1-4), optionally the raw moments.  Output planes are
-// row-major [ny][nx].
+// Fields of f(t) (steps 1-4), optionally the raw moments, written to the
+// caller's planes (row-major [ny][nx]).
 template <typename S, int QT, bool EX, int MODE>
 __global__ void __launch_bounds__(kThreads) k_fields(const __grid_constant__ Tables<S> tb,
                                                      const __grid_constant__ MomentArgs<S> a) {
@@ -875,25 +876,27 @@ __global__ void __launch_bounds__(kThreads) k_fields(const __grid_constant__ Tab
   moments9<S, QT, EX>(tb, a.s.Q, g, mm);
   const Macro M = landau<S>(a.s, mm);
   if (!M.ok) atomicAdd(a.status, 1ULL);
-  const long long P = a.s.ncell;
   const int cell = y * a.s.nx + x;
-  double* o = a.out;
-  o[0 * P + cell] = M.n;
-  o[1 * P + cell] = M.Ux / M.U0;
-  o[2 * P + cell] = M.Uy / M.U0;
-  o[3 * P + cell] = M.T;
-  o[4 * P + cell] = M.eps;
-  if (a.want_moments) {
-    o[5 * P + cell] = a.s.N0_ref + (double)mm[0];
-    o[6 * P + cell] = (double)mm[1];
-    o[7 * P + cell] = (double)mm[2];
-    o[8 * P + cell] = a.s.T00_ref + (double)mm[3];
-    o[9 * P + cell] = (double)mm[4];
-    o[10 * P + cell] = (double)mm[5];
-    o[11 * P + cell] = a.s.Tii_ref + (double)mm[6];
-    o[12 * P + cell] = (double)mm[7];
-    o[13 * P + cell] = a.s.Tii_ref + (double)mm[8];
+  double ux, uy;
+  if constexpr (sizeof(S) == 4) {      // (FP32 values: the FP64 quotients need no last ulp)
+    const double y = reciprocal(M.U0);
+    ux = M.Ux * y;
+    uy = M.Uy * y;
+  } else {
+    ux = M.Ux / M.U0;
+    uy = M.Uy / M.U0;
   }
+  const double f[5] = {M.n, ux, uy, M.T, M.eps};
+#pragma unroll
+  for (int k = 0; k < 5; ++k)
+    if (a.out[k]) a.out[k][cell] = f[k];
+  const double ref[9] = {a.s.N0_ref, 0.0, 0.0, a.s.T00_ref, 0.0, 0.0, a.s.Tii_ref, 0.0, a.s.Tii_ref};
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+    if (a.N) a.N[(size_t)j * a.s.ncell + cell] = ref[j] + (double)mm[j];
+#pragma unroll
+  for (int j = 3; j < 9; ++j)
+    if (a.Tab) a.Tab[(size_t)(j - 3) * a.s.ncell + cell] = ref[j] + (double)mm[j];
 }
 
 // Initialisation f*(0) = f^eq(n, U, T) (Sec. 6.2), stored shifted, with halo images.

@@ -9,7 +9,7 @@ import numpy as np
 import pytest
 
 from oracle import d3 as OD
-from tests.cases import rel_linf
+from tests.cases import oracle_quadrature, oracle_sim, permutation, rel_linf
 
 pytestmark = pytest.mark.gpu
 
@@ -74,4 +74,63 @@ def test_fields_of_fp32_storage_match_fp64_sums(rl, order):
         assert rel_linf(mo[name], w) <= 1e-13
     for k, name in ((1, "ux"), (2, "uy"), (3, "uz")):
         assert np.abs(mo[name] - want.u(k)).max() <= 1e-14
+    lat.close()
+
+
+def _state2(nx, ny, n0, T0, u0, seed):
+    rng = np.random.default_rng(seed)
+    y, x = np.meshgrid(*(2 * np.pi * np.arange(k) / k for k in (ny, nx)), indexing="ij")
+    p = rng.uniform(0, 2 * np.pi, 4)
+    n = n0 * (1 + 0.3 * np.cos(x + p[0]))
+    T = T0 * (1 + 0.1 * np.sin(y + p[1]))
+    return [np.ascontiguousarray(a) for a in (n, u0 * np.cos(y + p[2]), 0.5 * u0 * np.sin(x + p[3]), T)]
+
+
+@pytest.mark.parametrize("m,order,nx,ny,n0,T0,u0", [
+    (0.0, 2, 33, 5, 1.0, 1.0, 0.0), (0.0, 2, 200, 1, 1e-150, 1.3, 0.3), (0.0, 3, 3, 70, 2e100, 0.8, 0.4),
+    (0.0, 3, 65, 9, 1.0, 1.0, 0.6), (1.0, 2, 34, 6, 1.0, 1.1, 0.2), (5.0, 3, 33, 5, 1e8, 1.0, 0.2),
+    (10.0, 2, 31, 9, 1.0, 1.0, 0.1)])
+@pytest.mark.parametrize("stream", ["onlattice", "bilinear"])
+def test_fixed_point_step2_matches_oracle(rl, m, order, nx, ny, n0, T0, u0, stream):
+    lam = 1.0 if stream == "bilinear" else 0.0
+    lat = rl.Lattice(nx, ny, m=m, order=order, tau=0.8, precision="fp64", stream=stream, lam=lam)
+    quad = oracle_quadrature(m, order, lat.n, rl.plan(m=m, order=order)["v0"])
+    sim = oracle_sim(quad, nx, ny, tau=0.8, stream=stream, lam=lam or None)
+    fields = _state2(nx, ny, n0, T0, u0, order)
+    lat.init(*fields)
+    sim.init(*fields)
+    lat.step(2)
+    sim.step(2)
+    assert lat.sync_status() == (0, 0)
+    idx = permutation(lat.n, lat.p, quad)
+    assert rel_linf(lat.populations()[idx], sim.fs) <= 1e-12
+    mo = lat.moments(full=True)
+    assert rel_linf(mo["n"], sim.fields.n) <= 1e-12 and rel_linf(mo["T"], sim.fields.T) <= 1e-12
+    assert rel_linf(mo["N"], sim.fields.N) <= 1e-12
+    lat.close()
+
+
+@pytest.mark.parametrize("m,order", [(0.0, 2), (5.0, 3)])
+def test_cells_without_a_frame_are_counted_and_streamed(rl, m, order):
+    """A cell of negative density and one with an infinite population: both
+    counted, their finite populations streamed unrelaxed, an infinity turned NaN."""
+    nx, ny = 40, 11
+    lat = rl.Lattice(nx, ny, m=m, order=order, tau=0.9, precision="fp64")
+    lat.init(*_state2(nx, ny, 1.0, 1.0, 0.1, 3))
+    f = lat.populations()
+    f[:] = f[:, :1, :1]                            # uniform, so that streaming moves nothing
+    f[:, :, :] *= -1.0
+    lat.set_populations(f)
+    lat.step(1)
+    rc, count = lat.sync_status(raise_on_error=False)
+    assert rc == -4 and count == nx * ny
+    assert np.array_equal(lat.populations(), f)
+    f *= -1.0
+    f[3] = np.inf                                  # every cell pulls it
+    lat.set_populations(f)
+    lat.step(1)
+    rc, count = lat.sync_status(raise_on_error=False)
+    got = lat.populations()
+    assert rc == -4 and count == nx * ny
+    assert np.isnan(got[3]).all() and np.array_equal(np.delete(got, 3, 0), np.delete(f, 3, 0))
     lat.close()
