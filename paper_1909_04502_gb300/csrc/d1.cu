@@ -20,9 +20,10 @@
 // a copy of the end cell), so the pull reads base + x - s.  FP32 storage
 // holds g = f - f_ref (f_ref the equilibrium of (n_ref, rest, T_ref)) and
 // steps in FP32 from differences to that state (k_step1f); FP64 storage
-// steps in FP64 (Q <= 10 populations per cell).
+// steps in fixed point around an FP64 state (k_step1x; Q <= 10 populations per cell).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <memory>
@@ -31,6 +32,7 @@
 
 #include "../../include/rlbm.h"
 #include "dd.h"
+#include "fxstep.cuh"
 
 namespace rlbm1 {
 
@@ -72,7 +74,7 @@ struct Tab {
 struct Sc {
   int Q, N, nx, P;         // populations, order, cells, plane stride (nx + 2)
   int boundary;            // RLBM_BC_*
-  double tau;
+  double tau, inv_tau;
   double wall_T[2];        // equilibrium walls: first / last cell temperature (0: own T)
   double n_ref, T_ref;     // reference state of FP32 storage (n_ref = 0: none)
   double N0_ref, T00_ref;  // its moments: N^0 = n_ref, T^00 = T^xx = n_ref T_ref (eps = P)
@@ -100,47 +102,6 @@ __host__ __device__ inline void moments_dM(const Sc& s, double n, double U0, dou
     dM[2 * (a - 1)] = 0.5 * c * (Ea + Eia) - s.n_ref * fact * Trp;
     dM[2 * (a - 1) + 1] = 0.5 * c * (Ea - Eia);
   }
-}
-
-struct Macro1 {
-  double n, U0, Ux, T, eps, N0, Nx, T00, T0x;
-  bool ok;
-};
-
-// Steps 1-4 of Sec. 6.2 from the streamed populations (shifted by f_ref in
-// FP32 storage): moments, the Landau frame of the 2 x 2 mixed tensor
-// A = [[T00, -T0x], [T0x, -Txx]] (largest root of
-// l^2 - (T00 - Txx) l + T0x^2 - T00 Txx, eigenvector (Txx + l, T0x)),
-// n = U.N and T = eps / n.
-template <typename S>
-__device__ inline Macro1 macro1(const Tab<S>& tb, const Sc& s, const S* g) {
-  double N0 = 0.0, Nx = 0.0, T00 = 0.0, T0x = 0.0;
-  for (int i = 0; i < s.Q; ++i) {
-    const double f = (double)g[i], p = tb.p0[i];
-    const double fp = f * p;
-    N0 += fp;
-    T00 += fp * p;
-    if (tb.s[i] > 0) { Nx += fp; T0x += fp * p; }
-    else { Nx -= fp; T0x -= fp * p; }
-  }
-  Macro1 M;
-  M.N0 = s.N0_ref + N0;
-  M.Nx = Nx;
-  M.T00 = s.T00_ref + T00;
-  M.T0x = T0x;
-  const double Txx = M.T00;               // p^x p^x = p0 p0 on every population
-  const double disc = (M.T00 + Txx) * (M.T00 + Txx) - 4.0 * M.T0x * M.T0x;
-  const double l = 0.5 * ((M.T00 - Txx) + sqrt(fmax(disc, 0.0)));
-  const double v0 = Txx + l, v1 = M.T0x;
-  const double nu2 = v0 * v0 - v1 * v1;
-  const double inu = nu2 > 0.0 ? rsqrt(nu2) : 0.0;
-  M.U0 = v0 * inu;
-  M.Ux = v1 * inu;
-  M.eps = l;
-  M.n = M.U0 * M.N0 - M.Ux * M.Nx;
-  M.T = l / M.n;
-  M.ok = disc > 0.0 && nu2 > 0.0 && v0 > 0.0 && l > 0.0 && M.n > 0.0 && isfinite(M.T);
-  return M;
 }
 
 template <typename S>
@@ -171,35 +132,210 @@ __device__ inline void store1(const Sc& s, S* out, int i, int x, S v) {
   }
 }
 
-template <typename S>
-__global__ void __launch_bounds__(kThreads) k_step1(const __grid_constant__ Tab<S> tb, const __grid_constant__ Sc s,
-                                                    const S* __restrict__ fin, S* __restrict__ fout,
-                                                    unsigned long long* status) {
+// Store the Q values of cell x, and for an end cell its halo image (as
+// store1), the image stores behind one branch that interior warps skip.
+template <int Q, typename S>
+__device__ __forceinline__ void store_cell1(const Sc& s, S* out, int x, const S (&v)[Q]) {
+#pragma unroll
+  for (int i = 0; i < Q; ++i) out[(long long)i * s.P + x + 1] = v[i];
+  if (x == 0 || x == s.nx - 1) {
+    const bool per = s.boundary == RLBM_BC_PERIODIC;
+    if (x == 0) {
+      const int hx = per ? s.nx + 1 : 0;
+#pragma unroll
+      for (int i = 0; i < Q; ++i) out[(long long)i * s.P + hx] = v[i];
+    }
+    if (x == s.nx - 1) {
+      const int hx = per ? 0 : s.nx + 1;
+#pragma unroll
+      for (int i = 0; i < Q; ++i) out[(long long)i * s.P + hx] = v[i];
+    }
+  }
+}
+
+// FP64 storage, and the fields of both, with the population sums in 64-bit
+// fixed point (fx64.cuh).  In the light-cone sums A+- = sum p0 f, B+- = sum p0^2 f
+// over the two directions the frame is closed: T^00 +- T^0x = 2 B+- =
+// eps e^(+-2 theta), so eps = 2 sqrt(B+ B-), e^(4 theta) = B+ / B-,
+// n = e^(-theta) A+ + e^theta A- and T = eps / n; and as the even and odd entries
+// of a row of H agree, f^eq of direction s is sum_a H_ja (a-1)! m_a with
+// m_a = n T^(a-1) e^(s a theta) (with T / 2 and the powers of two in the table).
+// 35 FP64 operations per cell remain of 230 and still fill that pipe (2 per
+// clock and SM): 2^24 cells, order 3: 1.08 ms per step and for the fields
+// against 6.6 and 3.3 ms.
+constexpr int kBits1M = 62;            // populations in the moment sums (no sums of members)
+template <int N>
+struct Tab1x {
+  rlbm::Cx A[N], B[N], H[N][N];        // p0 2^(-ep - sk), p0^2 2^(-ep - sk), H (a-1)! 2^(a-1) 2^(-er - hk - rho)
+  int ep[N], er[N], rho[N], hk[N], skA, skB;
+  long long ref[N];                    // f_ref 2^ep in units of 2^(ref_E - kBits1M) (FP32 storage)
+  int ref_E;
+};
+
+struct Cell1 {
+  double A[2], B[2], eth[2], n;        // in units of 2^E; e^theta, e^-theta
+  double l2, T2;                       // eps / 2 (in units of 2^E), T / 2
+  int E;
+  bool ok;
+};
+
+template <int N, typename S>
+__device__ __forceinline__ Cell1 macro1x(const Tab1x<N>& tb, const S (&g)[2 * N]) {
+  using namespace rlbm;
+  long long mA[2], mB[2];
+  int Es[2];
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    mA[s] = mB[s] = 0;
+    long long X[N];
+    if constexpr (sizeof(S) == 8) {
+      int e = 0;
+      bool plain = true;
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        const int h = __double2hiint(g[2 * j + s]);
+        plain = plain && (unsigned)h < 0x7FF00000U;
+        e = max(e, ((h & 0x7FF00000) >> 20) + tb.ep[j]);
+      }
+      Es[s] = e + 1;
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        const double f = g[2 * j + s];
+        const int d = e - tb.ep[j];
+        if (__builtin_expect(plain, 1)) X[j] = to_fixed_cut<kBits1M>(f, d - (__double2hiint(f) >> 20));
+        else X[j] = to_fixed_any(f, d) << (kBits1M - kBits);
+      }
+    } else {
+      int e = tb.ref_E - 1;
+#pragma unroll
+      for (int j = 0; j < N; ++j) e = max(e, (int)((__float_as_uint(g[2 * j + s]) >> 23) & 0xFF) + 896 + 1 + tb.ep[j]);
+      Es[s] = e + 1;
+#pragma unroll
+      for (int j = 0; j < N; ++j)
+        X[j] = float_units(g[2 * j + s], e - tb.ep[j] - 896 + 63 - kBits1M) + (tb.ref[j] >> min(e + 1 - tb.ref_E, 63));
+    }
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      int h, l;
+      split_balanced(X[j], h, l);
+      add_product(mA[s], tb.A[j], h, l);
+      add_product(mB[s], tb.B[j], h, l);
+    }
+  }
+  Cell1 c;
+  c.E = max(Es[0], Es[1]);
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const int k = max(1023 - kBits1M + 64 - kCoefM + Es[s] - c.E, 1);
+    c.A[s] = from_fixed(mA[s], k + tb.skA);
+    c.B[s] = from_fixed(mB[s], k + tb.skB);
+  }
+  const double q = c.B[0] * c.B[1], r = reciprocal_sqrt(q), w = q * r;
+  c.l2 = fma(0.5 * r, fma(-w, w, q), w);
+  const double e2 = c.B[0] * r, y = reciprocal_sqrt(e2);
+  c.eth[0] = e2 * y;
+  c.eth[1] = y;
+  c.n = fma(c.eth[1], c.A[0], c.eth[0] * c.A[1]);
+  c.T2 = quotient(c.l2, c.n);
+  const float fB = fminf(cut_float(c.B[0]), cut_float(c.B[1])), fn = cut_float(c.n), fT = cut_float(c.T2);
+  c.ok = fB > 1e-30f && fn > 1e-30f && fn < 1e30f && fT > 1e-30f && fT < 1e30f && c.E > 128 &&
+         c.E < (sizeof(S) == 4 ? 1140 : 2040);
+  return c;
+}
+
+template <int N>
+__global__ void __launch_bounds__(kThreads) k_step1x(const __grid_constant__ Tab1x<N> tb, const __grid_constant__ Sc s,
+                                                     const double* __restrict__ fin, double* __restrict__ fout,
+                                                     unsigned long long* status) {
+  using namespace rlbm;
+  constexpr int Q = 2 * N;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= s.nx) return;
-  S g[kMaxQ];
-  for (int i = 0; i < s.Q; ++i) g[i] = fin[(long long)i * s.P + x + 1 - tb.s[i]];   // pull
-  const Macro1 M = macro1<S>(tb, s, g);
-  if (!M.ok) {
+  double g[Q];
+#pragma unroll
+  for (int i = 0; i < Q; ++i) g[i] = __ldg(fin + (long long)i * s.P + x + 2 * (i & 1));   // pull from x - s
+  Cell1 c = macro1x<N, double>(tb, g);
+  if (!c.ok) {
     atomicAdd(status, 1ULL);                                 // left unrelaxed (Omega = 0)
-    for (int i = 0; i < s.Q; ++i) store1<S>(s, fout, i, x, g[i]);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) g[i] = fma(0.0, -g[i], g[i]);
+    store_cell1<Q>(s, fout, x, g);
     return;
   }
-  double dM[kMaxQ];
-  const bool wall = s.boundary == RLBM_BC_EQWALL_X && (x == 0 || x == s.nx - 1);
-  if (wall) {
-    const double Tw = s.wall_T[x == 0 ? 0 : 1] > 0.0 ? s.wall_T[x == 0 ? 0 : 1] : M.T;
-    moments_dM(s, M.n, 1.0, 0.0, Tw, dM);
-    for (int i = 0; i < s.Q; ++i) store1<S>(s, fout, i, x, feq_i<S>(tb, s, i, dM));
-    return;
+  double om[2] = {s.inv_tau * c.eth[1], s.inv_tau * c.eth[0]};   // p.U / (p0 tau)
+  if (s.boundary == RLBM_BC_EQWALL_X && (x == 0 || x == s.nx - 1)) {
+    // f^eq(n, rest, T_w), T_w the prescribed wall temperature or the cell's own, unrelaxed
+    const double Tw = s.wall_T[x == 0 ? 0 : 1];
+    c.T2 = Tw > 0.0 ? 0.5 * Tw : c.T2;
+    c.eth[0] = c.eth[1] = om[0] = om[1] = 1.0;
   }
-  moments_dM(s, M.n, M.U0, M.Ux, M.T, dM);
-  const double itau = 1.0 / s.tau;
-  for (int i = 0; i < s.Q; ++i) {
-    const S om = (S)((M.U0 - (double)tb.s[i] * M.Ux) * itau);   // p.U / (p0 tau)
-    const S fe = feq_i<S>(tb, s, i, dM);
-    store1<S>(s, fout, i, x, g[i] + om * (fe - g[i]));
+  const int xo = above(fmaxf(cut_float(om[0]), cut_float(om[1]))), eo = max(xo, -2), uf = max(0, xo - 2);
+  const long long half = 1LL << (29 - eo);
+#pragma unroll
+  for (int d = 0; d < 2; ++d) {
+    double m[N];
+    const double z = c.T2 * c.eth[d];
+    m[0] = c.n * c.eth[d];
+    float sum = cut_float(m[0]) * __uint_as_float((unsigned)(127 + tb.hk[0]) << 23);
+#pragma unroll
+    for (int a = 1; a < N; ++a) {
+      m[a] = m[a - 1] * z;
+      sum += cut_float(m[a]) * __uint_as_float((unsigned)(127 + tb.hk[a]) << 23);
+    }
+    const int xg = above(sum), sE = c.E + xg, ue = sE + max(0, xo - 3);
+    int vh[N], vl[N];
+#pragma unroll
+    for (int a = 0; a < N; ++a) {
+      split_balanced(to_fixed_cut<62>(m[a], xg + 1022 - tb.hk[a] - (__double2hiint(m[a]) >> 20)), vh[a], vl[a]);
+    }
+    int oh, ol;
+    split_balanced(to_fixed_cut<62>(om[d], eo + 1022 - (__double2hiint(om[d]) >> 20)), oh, ol);
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const int i = 2 * j + d;
+      Acc h{0, 0x80000000LL};
+#pragma unroll
+      for (int a = 0; a < N; ++a) macs(h, tb.H[j][a], vh[a], vl[a]);
+      const int hi = __double2hiint(g[i]), e = (hi & 0x7FF00000) >> 20;
+      const int u = max(e + 1 - tb.er[j] + uf, tb.rho[j] + ue), sh = min(u - tb.rho[j] - sE, 62);
+      const long long C = (h.H + (long long)hi32(h.M) + ((1LL << sh) >> 1)) >> sh;
+      const int dd = u - 1 + tb.er[j] - e;
+      long long X = __builtin_expect(hi >= 0, 1) ? to_fixed_positive(g[i], dd) : to_fixed_any(g[i], dd + e);
+      int dh, dl;
+      split_balanced(C - X, dh, dl);
+      Acc q{0, half};
+      macs(q, Cx{oh, ol}, dh, dl);
+      X += collect(q, 2 + eo);
+      const int k = u + tb.er[j] - kBits;
+      g[i] = __builtin_expect(hi32(X) > 0, 1) ? from_fixed_positive(X, k) : from_fixed_any(X, k);
+    }
   }
+  store_cell1<Q>(s, fout, x, g);
+}
+
+// Fields of the streamed populations (pull = 1) or of the stored ones:
+// out[8][nx] = n, ux, T, eps, N0, Nx, T00, T0x (n NaN without a Landau frame).
+template <int N, typename S>
+__global__ void __launch_bounds__(kThreads) k_fields1x(const __grid_constant__ Tab1x<N> tb, const __grid_constant__ Sc s,
+                                                       const S* __restrict__ fin, int pull, double* out) {
+  using namespace rlbm;
+  constexpr int Q = 2 * N;
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  if (x >= s.nx) return;
+  S g[Q];
+#pragma unroll
+  for (int i = 0; i < Q; ++i) g[i] = __ldg(fin + (long long)i * s.P + x + (pull ? 2 * (i & 1) : 1));
+  const Cell1 c = macro1x<N, S>(tb, g);
+  const int nx = s.nx, k = c.E - 1023;
+  const double T00 = c.B[0] + c.B[1], T0x = c.B[0] - c.B[1];
+  out[x] = c.ok ? scaled(c.n, k) : __longlong_as_double(0x7ff8000000000000LL);
+  out[nx + x] = T0x * reciprocal(fma(2.0, c.l2, T00));
+  out[2 * nx + x] = 2.0 * c.T2;
+  out[3 * nx + x] = scaled(c.l2, k + 1);
+  out[4 * nx + x] = scaled(c.A[0] + c.A[1], k);
+  out[5 * nx + x] = scaled(c.A[0] - c.A[1], k);
+  out[6 * nx + x] = scaled(T00, k);
+  out[7 * nx + x] = scaled(T0x, k);
 }
 
 // FP32 storage (g = f - f_ref): the step in FP32 throughout, with every
@@ -217,7 +353,7 @@ __global__ void __launch_bounds__(kThreads) k_step1(const __grid_constant__ Tab<
 //                       + n_ref (T^(a-1) - T_ref^(a-1)),
 //   dM_{a,1} / (a-1)! = n T^(a-1) (E_th^a - 1)(E_th^a + 1) / (2 E_th^a),
 // T^(a-1) - T_ref^(a-1) = T (T^(a-2) - T_ref^(a-2)) + T_ref^(a-2) dT.
-// The FP64-storage step (k_step1<double>) keeps the FP64 arithmetic.
+// The FP64-storage step is k_step1x.
 template <int N>
 __device__ __forceinline__ void moments_dM_f32(float n, float dn, float T, float dT, float Em1, float Eth,
                                                float nr, float Tr, float (&dM)[2 * N]) {
@@ -236,27 +372,6 @@ __device__ __forceinline__ void moments_dM_f32(float n, float dn, float T, float
     const float h = __fdividef(0.5f * n * Ta * Em1a, Ea);
     dM[2 * (a - 1)] = fact * (h * Em1a + dn * Ta + nr * DTa);
     dM[2 * (a - 1) + 1] = fact * h * (Ea + 1.f);
-  }
-}
-
-// Store the Q values of cell x, and for an end cell its halo image (as
-// store1), the image stores behind one branch that interior warps skip.
-template <int Q>
-__device__ __forceinline__ void store_cell1f(const Sc& s, float* out, int x, const float (&v)[Q]) {
-#pragma unroll
-  for (int i = 0; i < Q; ++i) out[(long long)i * s.P + x + 1] = v[i];
-  if (x == 0 || x == s.nx - 1) {
-    const bool per = s.boundary == RLBM_BC_PERIODIC;
-    if (x == 0) {
-      const int hx = per ? s.nx + 1 : 0;
-#pragma unroll
-      for (int i = 0; i < Q; ++i) out[(long long)i * s.P + hx] = v[i];
-    }
-    if (x == s.nx - 1) {
-      const int hx = per ? 0 : s.nx + 1;
-#pragma unroll
-      for (int i = 0; i < Q; ++i) out[(long long)i * s.P + hx] = v[i];
-    }
   }
 }
 
@@ -321,7 +436,7 @@ __device__ __forceinline__ void cell1f(const Tab<float>& tb, const Sc& s, const 
                   isfinite(U0) && isfinite(dn);
   if (!ok) {
     atomicAdd(status, 1ULL);                                 // left unrelaxed (Omega = 0)
-    store_cell1f<Q>(s, fout, x, g);
+    store_cell1<Q>(s, fout, x, g);
     return;
   }
   // f^eq of the pair (shell j, +1), (shell j, -1) from the first row: the
@@ -347,7 +462,7 @@ __device__ __forceinline__ void cell1f(const Tab<float>& tb, const Sc& s, const 
     moments_dM_f32<N>(n, dn, Tw, dTw, 0.f, 1.f, nr, Tr, dM);
 #pragma unroll
     for (int j = 0; j < N; ++j) feq_pair(j, dM, o[2 * j], o[2 * j + 1]);
-    store_cell1f<Q>(s, fout, x, o);
+    store_cell1<Q>(s, fout, x, o);
     return;
   }
   const float Em1 = Ux + __fdividef(Ux * Ux, U0 + 1.f);     // e^theta - 1
@@ -361,7 +476,7 @@ __device__ __forceinline__ void cell1f(const Tab<float>& tb, const Sc& s, const 
     o[2 * j] = fmaf(omp, fp - g[2 * j], g[2 * j]);
     o[2 * j + 1] = fmaf(omm, fm - g[2 * j + 1], g[2 * j + 1]);
   }
-  store_cell1f<Q>(s, fout, x, o);
+  store_cell1<Q>(s, fout, x, o);
 }
 
 // CPT cells per thread, kThreads apart: every thread issues the pulls of
@@ -404,27 +519,6 @@ __global__ void __launch_bounds__(kThreads) k_init1(const __grid_constant__ Tab<
   double dM[kMaxQ];
   moments_dM(s, n[x], gam, gam * u, T[x], dM);
   for (int i = 0; i < s.Q; ++i) store1<S>(s, fout, i, x, feq_i<S>(tb, s, i, dM));
-}
-
-// Fields of the streamed populations (pull = 1) or of the stored ones:
-// out[8][nx] = n, ux, T, eps, N0, Nx, T00, T0x (n NaN without a Landau frame).
-template <typename S>
-__global__ void __launch_bounds__(kThreads) k_fields1(const __grid_constant__ Tab<S> tb, const __grid_constant__ Sc s,
-                                                      const S* __restrict__ fin, int pull, double* out) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= s.nx) return;
-  S g[kMaxQ];
-  for (int i = 0; i < s.Q; ++i) g[i] = fin[(long long)i * s.P + x + 1 - (pull ? tb.s[i] : 0)];
-  const Macro1 M = macro1<S>(tb, s, g);
-  const int nx = s.nx;
-  out[x] = M.ok ? M.n : __longlong_as_double(0x7ff8000000000000LL);
-  out[nx + x] = M.Ux / M.U0;
-  out[2 * nx + x] = M.T;
-  out[3 * nx + x] = M.eps;
-  out[4 * nx + x] = M.N0;
-  out[5 * nx + x] = M.Nx;
-  out[6 * nx + x] = M.T00;
-  out[7 * nx + x] = M.T0x;
 }
 
 // Host: the order-N table and H = inverse of phi_{a,b}(p_i) in double-double.
@@ -491,6 +585,11 @@ struct rlbm1_handle {
   Sc sc{};
   std::unique_ptr<Tab<float>> tf;
   std::unique_ptr<Tab<double>> td;
+  // fixed-point tables of the order in use (the FP64 step, the fields)
+  std::unique_ptr<Tab1x<2>> tx2;
+  std::unique_ptr<Tab1x<3>> tx3;
+  std::unique_ptr<Tab1x<4>> tx4;
+  std::unique_ptr<Tab1x<5>> tx5;
   std::vector<double> p0, w, fref;
   std::vector<int> sgn;
   size_t elem = 8;
@@ -540,6 +639,70 @@ void fill(const rlbm1_handle* h, const std::vector<double>& H, Tab<S>* t) {
       t->H[i][k] = H[(size_t)i * Q + k];
       t->Hs[i][k] = (S)H[(size_t)i * Q + k];
     }
+  }
+}
+
+// The fixed-point tables of the FP64 step and of the fields; false where a row's
+// even and odd entries differ (the built-in tables' agree exactly).
+template <int N>
+bool fill1x(const rlbm1_handle* h, const std::vector<double>& H, Tab1x<N>* t) {
+  std::memset(t, 0, sizeof(Tab1x<N>));
+  auto row = [&](int j, int a) {
+    double f = 1.0;
+    for (int k = 2; k <= a; ++k) f *= k;
+    return std::ldexp(H[(size_t)2 * j * 2 * N + 2 * a] * f, a);      // H 2^(a-1) (a-1)!, a counted from 0 here
+  };
+  double sA = 0.0, sB = 0.0;
+  int e = -1000;
+  for (int j = 0; j < N; ++j) {
+    double rest = 0.0;
+    for (int a = 0; a < N; ++a) {
+      if (H[(size_t)2 * j * 2 * N + 2 * a] != H[(size_t)2 * j * 2 * N + 2 * a + 1]) return false;
+      rest += std::ldexp(row(j, a), -a);
+    }
+    if (!(rest > 0.0)) return false;
+    const double p = h->p0[2 * j], r = h->fref[2 * j];
+    t->er[j] = std::ilogb(rest);
+    t->ep[j] = std::ilogb(p * p);
+    sA += std::ldexp(p, -t->ep[j]);
+    sB += std::ldexp(p * p, -t->ep[j]);
+    if (r != 0.0) e = std::max(e, std::ilogb(r) + t->ep[j] + 1);
+  }
+  std::frexp(sA, &t->skA);
+  std::frexp(sB, &t->skB);
+  t->ref_E = 1023 + e + 1;
+  for (int a = 0; a < N; ++a) {
+    double big = 0.0;
+    for (int j = 0; j < N; ++j) big = std::fmax(big, std::fabs(std::ldexp(row(j, a), -t->er[j])));
+    std::frexp(big, &t->hk[a]);
+  }
+  for (int j = 0; j < N; ++j) {
+    const double p = h->p0[2 * j], r = h->fref[2 * j];
+    double big = 0.0, sum = 0.0;
+    for (int a = 0; a < N; ++a) {
+      const double v = std::fabs(std::ldexp(row(j, a), -t->er[j] - t->hk[a]));
+      big = std::fmax(big, v);
+      sum += v;
+    }
+    std::frexp(big, &t->rho[j]);
+    if (!(std::ldexp(sum, -t->rho[j]) <= 4.0)) return false;
+    for (int a = 0; a < N; ++a)
+      t->H[j][a] = rlbm::split_constant(std::ldexp(row(j, a), -t->er[j] - t->hk[a] - t->rho[j]), rlbm::kCoefH);
+    t->A[j] = rlbm::split_constant(std::ldexp(p, -t->ep[j] - t->skA), rlbm::kCoefM);
+    t->B[j] = rlbm::split_constant(std::ldexp(p * p, -t->ep[j] - t->skB), rlbm::kCoefM);
+    t->ref[j] = r == 0.0 ? 0 : std::llround(std::ldexp(r, t->ep[j] + kBits1M - (t->ref_E - 1023)));
+  }
+  return true;
+}
+
+// f(table) with the handle's table of order N
+template <typename F>
+void with_tab1x(const rlbm1_handle* h, F&& f) {
+  switch (h->sc.N) {
+    case 2: f(*h->tx2); break;
+    case 3: f(*h->tx3); break;
+    case 4: f(*h->tx4); break;
+    default: f(*h->tx5); break;
   }
 }
 
@@ -593,6 +756,7 @@ int rlbm1_create(int nx, int order, double tau, int boundary, const double* wall
   s.P = nx + 2;
   s.boundary = boundary;
   s.tau = tau;
+  s.inv_tau = 1.0 / tau;
   s.wall_T[0] = wall_T ? wall_T[0] : 0.0;
   s.wall_T[1] = wall_T ? wall_T[1] : 0.0;
   s.n_ref = precision == RLBM_FP32_STORE ? 1.0 : 0.0;
@@ -621,6 +785,14 @@ int rlbm1_create(int nx, int order, double tau, int boundary, const double* wall
   }
   if (h->elem == 4) { h->tf.reset(new Tab<float>()); fill(h.get(), H, h->tf.get()); }
   else { h->td.reset(new Tab<double>()); fill(h.get(), H, h->td.get()); }
+  bool fx = false;
+  switch (order) {
+    case 2: h->tx2.reset(new Tab1x<2>()); fx = fill1x(h.get(), H, h->tx2.get()); break;
+    case 3: h->tx3.reset(new Tab1x<3>()); fx = fill1x(h.get(), H, h->tx3.get()); break;
+    case 4: h->tx4.reset(new Tab1x<4>()); fx = fill1x(h.get(), H, h->tx4.get()); break;
+    default: h->tx5.reset(new Tab1x<5>()); fx = fill1x(h.get(), H, h->tx5.get()); break;
+  }
+  if (!fx) return fail1(nullptr, RLBM_ERR_QUADRATURE, "1-d equilibrium matrix without the direction symmetry");
   const size_t bytes = (size_t)s.Q * s.P * h->elem;
   for (int b = 0; b < 2; ++b)
     if (cudaMalloc(&h->buf[b], bytes) != cudaSuccess) { cudaGetLastError(); return fail1(nullptr, RLBM_ERR_OOM, "population buffers"); }
@@ -697,8 +869,10 @@ int rlbm1_step(rlbm1_handle* h, int nsteps) {
         default: k_step1f<5, kStep1CPT><<<gr, kThreads, 0, h->stream>>>(*h->tf, h->sc, in, o, h->status); break;
       }
     } else
-      k_step1<double><<<grid1(h->sc.nx), kThreads, 0, h->stream>>>(*h->td, h->sc, (const double*)h->buf[h->cur],
-                                                                    (double*)h->buf[h->cur ^ 1], h->status);
+      with_tab1x(h, [&](const auto& t) {
+        k_step1x<<<grid1(h->sc.nx), kThreads, 0, h->stream>>>(t, h->sc, (const double*)h->buf[h->cur],
+                                                              (double*)h->buf[h->cur ^ 1], h->status);
+      });
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail1(h, e, "rlbm1_step");
     h->cur ^= 1;
@@ -713,10 +887,10 @@ int rlbm1_moments(rlbm1_handle* h, double* out, int on_device) {
   const void* src = h->have_prev ? h->buf[h->cur ^ 1] : h->buf[h->cur];
   const int pull = h->have_prev ? 1 : 0;
   double* dst = on_device ? out : h->fields;
-  if (h->elem == 4)
-    k_fields1<float><<<grid1(nx), kThreads, 0, h->stream>>>(*h->tf, h->sc, (const float*)src, pull, dst);
-  else
-    k_fields1<double><<<grid1(nx), kThreads, 0, h->stream>>>(*h->td, h->sc, (const double*)src, pull, dst);
+  with_tab1x(h, [&](const auto& t) {
+    if (h->elem == 4) k_fields1x<<<grid1(nx), kThreads, 0, h->stream>>>(t, h->sc, (const float*)src, pull, dst);
+    else k_fields1x<<<grid1(nx), kThreads, 0, h->stream>>>(t, h->sc, (const double*)src, pull, dst);
+  });
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && !on_device) {
     e = cudaMemcpyAsync(out, h->fields, sizeof(double) * 8 * nx, cudaMemcpyDeviceToHost, h->stream);

@@ -50,6 +50,27 @@ __device__ __forceinline__ int run_exponent(const double (&f)[L], bool& plain) {
 __device__ __noinline__ long long to_fixed_any(double f, int d) { return to_fixed(f, d - biased_exponent(f)); }
 __device__ __noinline__ double from_fixed_any(long long Y, int k) { return from_fixed(Y, k); }
 
+// g 2^ep (a float, exact) in units of 2^(E - BITS): d = E - 1 - ep - 896 + 63 - BITS.
+__device__ __forceinline__ long long float_units(float g, int d) {
+  const unsigned b = __float_as_uint(g);
+  const int v = (int)((b & 0x7FFFFFU) | 0x800000U), s = (int)b >> 31;
+  long long x = (long long)(((unsigned long long)(unsigned)(((v ^ s) - s) << 7)) << 32);
+  asm("shr.s64 %0, %0, %1;" : "+l"(x) : "r"(d - (int)((b >> 23) & 0xFF)));
+  return x;
+}
+
+// v 2^k, the exponent raised in place where the result is normal
+__device__ __noinline__ double scaled_any(double v, int k) {
+  const int k1 = k / 2;
+  return v * __hiloint2double((1023 + k1) << 20, 0) * __hiloint2double((1023 + k - k1) << 20, 0);
+}
+__device__ __forceinline__ double scaled(double v, int k) {
+  const int h = __double2hiint(v), e = (h >> 20) & 0x7FF;
+  if (__builtin_expect(e > 0 && e < 0x7FF && e + k > 0 && e + k < 0x7FF, 1))
+    return __hiloint2double(h + (k << 20), __double2loint(v));
+  return scaled_any(v, k);
+}
+
 // Values of a thread split for products (split_balanced), in a shared-memory
 // column of its own: in registers they would hold 28 to 76 of them.
 struct Column {

@@ -491,19 +491,17 @@ __global__ void __launch_bounds__(kThreads2x) k_fields2x(const __grid_constant__
   const bool ok = c.ok && E > 128 && E < 2040;
   if (!ok) atomicAdd(a.status, 1ULL);
   const int cell = y * s.nx + x;
-  // 2^(E - 1023) in two factors (E may lie outside the exponent's range)
-  const int e1 = E / 2, e2 = E - e1;
-  const double s1 = __hiloint2double((e1 + 512) << 20, 0), s2 = __hiloint2double((e2 + 511) << 20, 0);
-  const double f[5] = {c.n * s1 * s2, c.u[0], c.u[1], c.T, c.L * s1 * s2};
+  const int k2 = E - 1023;
+  const double f[5] = {scaled(c.n, k2), c.u[0], c.u[1], c.T, scaled(c.L, k2)};
 #pragma unroll
   for (int k = 0; k < 5; ++k)
     if (a.out[k]) a.out[k][cell] = f[k];
 #pragma unroll
   for (int j = 0; j < 3; ++j)
-    if (a.N) a.N[(size_t)j * s.ncell + cell] = v[j] * s1 * s2;
+    if (a.N) a.N[(size_t)j * s.ncell + cell] = scaled(v[j], k2);
 #pragma unroll
   for (int j = 0; j < 6; ++j)
-    if (a.Tab) a.Tab[(size_t)j * s.ncell + cell] = v[3 + j] * s1 * s2;
+    if (a.Tab) a.Tab[(size_t)j * s.ncell + cell] = scaled(v[3 + j], k2);
 }
 
 template <int MODE, bool MASSLESS>

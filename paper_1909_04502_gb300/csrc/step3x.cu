@@ -93,13 +93,7 @@ __device__ __forceinline__ void run_units(const float (&g)[L], int ep, long long
   const int d = E - 1 - ep - 896 + 63 - kBitsM;
   const long long r = ref >> min(E - ref_E, 63);
 #pragma unroll
-  for (int q = 0; q < L; ++q) {
-    const unsigned b = __float_as_uint(g[q]);
-    const int v = (int)((b & 0x7FFFFFU) | 0x800000U), s = (int)b >> 31;
-    long long x = (long long)(((unsigned long long)(unsigned)(((v ^ s) - s) << 7)) << 32);
-    asm("shr.s64 %0, %0, %1;" : "+l"(x) : "r"(d - (int)((b >> 23) & 0xFF)));
-    X[q] = x + r;
-  }
+  for (int q = 0; q < L; ++q) X[q] = float_units(g[q], d) + r;
 }
 
 // The macroscopic state of a cell in units of 2^E: eps U^a = T^ab U_b with
@@ -481,16 +475,13 @@ __global__ void __launch_bounds__(128) k_fields3x(const __grid_constant__ Tables
   moment_values(m, tb.sk, N, T00, t, Sm);
   const Cell3 c = landau3x(N, T00, t, Sm);
   const bool ok = c.ok && E > 128 && E < (sizeof(S) == 4 ? 1140 : 2040);   // (an infinity or NaN lies above)
-  // 2^(E - 1023) in two factors (E may be outside the exponent's range)
-  const int e1 = E / 2, e2 = E - e1;
-  const double s1 = __hiloint2double((e1 + 512) << 20, 0), s2 = __hiloint2double((e2 + 511) << 20, 0);
   const long long cell = ((long long)z * s.ny + y) * s.nx + x, nc = (long long)s.nx * s.ny * s.nz;
-  a.out[cell] = ok ? c.n * s1 * s2 : __longlong_as_double(0x7ff8000000000000LL);
+  a.out[cell] = ok ? scaled(c.n, E - 1023) : __longlong_as_double(0x7ff8000000000000LL);
   a.out[nc + cell] = c.u[0];
   a.out[2 * nc + cell] = c.u[1];
   a.out[3 * nc + cell] = c.u[2];
   a.out[4 * nc + cell] = quotient(third(c.L), c.n);
-  a.out[5 * nc + cell] = c.L * s1 * s2;
+  a.out[5 * nc + cell] = scaled(c.L, E - 1023);
 }
 
 dim3 grid3x(const Scalars3& s) { return dim3((s.nx + 31) / 32, (s.ny + 3) / 4, s.nz); }

@@ -134,3 +134,32 @@ def test_cells_without_a_frame_are_counted_and_streamed(rl, m, order):
     assert rc == -4 and count == nx * ny
     assert np.isnan(got[3]).all() and np.array_equal(np.delete(got, 3, 0), np.delete(f, 3, 0))
     lat.close()
+
+
+@pytest.mark.parametrize("order", [2, 3, 5])
+@pytest.mark.parametrize("nx,n0,T0,u0,boundary", [(1, 1.0, 1.0, 0.0, "periodic"), (129, 1e-140, 1.0, 0.3, "periodic"),
+                                                  (257, 1e90, 0.6, 0.6, "freeflow_x"), (40, 1.0, 1.5, 0.2, "eqwall_x")])
+def test_fixed_point_step1_matches_oracle(rl, order, nx, n0, T0, u0, boundary):
+    """The (1+1)-d step: f and the fields against the oracle.  At order 5 the
+    equilibrium's condition number reaches 2^13 off the reference temperature,
+    in the oracle's FP64 sums as in the step: 1e-11 there."""
+    from oracle import d1 as O1
+    x = 2 * np.pi * np.arange(nx) / nx
+    fields = [np.ascontiguousarray(a) for a in (n0 * (1 + 0.2 * np.sin(x)), u0 * np.cos(x + 0.4) + 0 * x,
+                                                T0 * (1 + 0.1 * np.cos(x)))]
+    lat = rl.Lattice1(nx, order=order, tau=0.8, boundary=boundary, precision="fp64")
+    sim = O1.Simulation1(O1.massless_quadrature_1d(order), nx, tau=0.8, boundary=boundary)
+    lat.init(*fields)
+    sim.init(*fields)
+    lat.step(2)
+    sim.step(2)
+    assert lat.sync_status() == (0, 0)
+    tol = 1e-12 if order < 5 else 1e-11
+    q = sim.quad
+    pos = {(int(s), round(float(p), 9)): i for i, (s, p) in enumerate(zip(lat.n, lat.p[:, 0]))}
+    idx = [pos[(int(s), round(float(p), 9))] for s, p in zip(q.n, q.p[:, 0])]
+    assert rel_linf(lat.populations()[idx], sim.fs) <= tol
+    mo = lat.moments()
+    assert rel_linf(mo["n"], sim.fields.n) <= tol and rel_linf(mo["T"], sim.fields.T) <= tol
+    assert rel_linf(mo["eps"], sim.fields.eps) <= tol
+    lat.close()
