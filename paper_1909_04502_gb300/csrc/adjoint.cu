@@ -362,8 +362,15 @@ __global__ void __launch_bounds__(kThreads, (sizeof(S) == 4 ? 640 : 256) / kThre
   });
 }
 
+// The loss, a count of finished blocks, and from kLossParts on the sum of each block.
+constexpr int kLossParts = 2;
+inline size_t loss_bytes(const Scalars& s) {
+  const dim3 g = grid_for(s);
+  return (kLossParts + (size_t)g.x * g.y) * sizeof(double);
+}
+
 // Loss L = 1/2 sum_x |u(x) - u_target(x)|^2 on the fields of f(T) = S x(T-1):
-// writes a(T) = dL/df(T) and adds L to *loss.
+// writes a(T) = dL/df(T) and L to loss[0] (the first kLossParts entries zero before).
 template <typename S>
 struct AdjLossArgs {
   Scalars s;
@@ -424,13 +431,32 @@ __global__ void __launch_bounds__(kThreads) k_adj_loss(const __grid_constant__ T
         if (i < Qn) hb[i * a.s.iplane] = out[i];
     });
   }
-  s_red[tid] = part;
-  __syncthreads();
-  for (int w = kThreads / 2; w > 0; w >>= 1) {
-    if (tid < w) s_red[tid] += s_red[tid + w];
+  auto total = [&](double v) {
+    s_red[tid] = v;
     __syncthreads();
+    for (int w = kThreads / 2; w > 0; w >>= 1) {
+      if (tid < w) s_red[tid] += s_red[tid + w];
+      __syncthreads();
+    }
+    return s_red[0];
+  };
+  // The block that comes last adds the blocks' sums in their order, so that the
+  // loss does not depend on how the blocks fall beside the recomputation's.
+  __shared__ bool s_last;
+  const int blocks = gridDim.x * gridDim.y;
+  const double mine = total(part);
+  if (tid == 0) {
+    a.loss[kLossParts + blockIdx.y * gridDim.x + blockIdx.x] = mine;
+    __threadfence();
+    s_last = atomicAdd((unsigned*)(a.loss + 1), 1u) == (unsigned)blocks - 1;
   }
-  if (tid == 0) atomicAdd(a.loss, s_red[0]);
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  double sum = 0.0;
+  for (int b = tid; b < blocks; b += kThreads) sum += __ldcg(a.loss + kLossParts + b);
+  const double all = total(sum);
+  if (tid == 0) a.loss[0] = all;
 }
 
 // Initial state x(0) = f_ref + H dM(n0, U(u0), T0): dL/du0 from lambda(0) = S^T a(1).
@@ -632,7 +658,7 @@ int rlbm_adjoint_create(rlbm_handle* h, int nsteps, int checkpoint_every, rlbm_a
   if (e == cudaSuccess) e = cudaMalloc(&A->adj[1], A->buf_bytes);
   if (e == cudaSuccess) e = cudaMalloc(&A->gtau, nc * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&A->init_fields, 4 * nc * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&A->loss, sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc(&A->loss, loss_bytes(h->sc));
   if (e != cudaSuccess) {
     cudaGetLastError();
     free_adjoint(A.get());
@@ -713,7 +739,7 @@ int rlbm_adjoint_backward(rlbm_adjoint* A, const double* ux_target, const double
     uyt = h->fields + nc;
   }
   cudaMemsetAsync(A->gtau, 0, nc * sizeof(double), st);
-  cudaMemsetAsync(A->loss, 0, sizeof(double), st);
+  cudaMemsetAsync(A->loss, 0, kLossParts * sizeof(double), st);
   int an = 0;                  // adj[an] holds a(t+1)
   bool have_a = false;
   // Segment sgi covers the states x(c) .. x(last), c = sgi K.  Its adjoint
