@@ -336,6 +336,7 @@ struct AdjArgs {
 template <typename S, int QT, bool EX, int MODE, bool SYM, bool MIN>
 __global__ void __launch_bounds__(kThreads, (sizeof(S) == 4 ? 640 : 256) / kThreads) k_adj_step(const __grid_constant__ Tables<S> tb,
                                                        const __grid_constant__ AdjArgs<S> a) {
+  const S* const anext = chain_begin(a.anext);
   const int x = blockIdx.x * kBX + threadIdx.x;
   const int y = blockIdx.y * kBY + threadIdx.y;
   if (x >= a.s.nx || y >= a.s.ny) return;
@@ -343,11 +344,11 @@ __global__ void __launch_bounds__(kThreads, (sizeof(S) == 4 ? 640 : 256) / kThre
   const int cell = y * a.s.nx + x;
   const int Qn = EX ? QT : a.s.Q;
   S g[QT], lam[QT], out[QT];
-  gather<S, QT, EX, MODE>(tb, a.s, a.xprev, si, g);
-  gather_rev<S, QT, EX, MODE>(tb, a.s, a.anext, si, lam);
-  const S tau = (a.s.tau_mode == 1) ? a.tau_field[cell] : const_tau<S>(a.s);
+  gather<S, QT, EX, MODE>(tb, a.s, chained(a.xprev), si, g);
+  gather_rev<S, QT, EX, MODE>(tb, a.s, anext, si, lam);
+  const S tau = (a.s.tau_mode == 1) ? chained(a.tau_field)[cell] : const_tau<S>(a.s);
   S gt;
-  collide_vjp<S, QT, EX, SYM, MIN>(tb, a.s, g, lam, tau, out, gt, a.status, a.macro, cell);
+  collide_vjp<S, QT, EX, SYM, MIN>(tb, a.s, g, lam, tau, out, gt, a.status, chained(a.macro), cell);
   if constexpr (sizeof(S) == 4) a.gtau[cell] += f2d(gt);   // exact conversion on the integer pipe
   else a.gtau[cell] += gt;
   S* __restrict__ ob = a.aout + si;
@@ -508,15 +509,15 @@ template <typename S, int QT, bool EX, bool SYM>
 cudaError_t adj_step_q(const Tables<S>& tb, const AdjArgs<S>& a, int mode, cudaStream_t st) {
   if constexpr (SYM && sizeof(S) == 4) {
     if (a.macro) {
-      if (mode == kOnLattice) k_adj_step<S, QT, EX, kOnLattice, SYM, true><<<grid_for(a.s), block_dim(), 0, st>>>(tb, a);
-      else k_adj_step<S, QT, EX, kBilinear, SYM, true><<<grid_for(a.s), block_dim(), 0, st>>>(tb, a);
-      return cudaGetLastError();
+      return launch_chained(true, mode == kOnLattice ? k_adj_step<S, QT, EX, kOnLattice, SYM, true>
+                                               : k_adj_step<S, QT, EX, kBilinear, SYM, true>,
+                            grid_for(a.s), block_dim(), 0, st, tb, a);
     }
   }
   if (a.macro) return cudaErrorInvalidValue;
-  if (mode == kOnLattice) k_adj_step<S, QT, EX, kOnLattice, SYM, false><<<grid_for(a.s), block_dim(), 0, st>>>(tb, a);
-  else k_adj_step<S, QT, EX, kBilinear, SYM, false><<<grid_for(a.s), block_dim(), 0, st>>>(tb, a);
-  return cudaGetLastError();
+  return launch_chained(true, mode == kOnLattice ? k_adj_step<S, QT, EX, kOnLattice, SYM, false>
+                                           : k_adj_step<S, QT, EX, kBilinear, SYM, false>,
+                        grid_for(a.s), block_dim(), 0, st, tb, a);
 }
 
 // the built-in massless stencil (orbit order, exactly symmetric H) takes the

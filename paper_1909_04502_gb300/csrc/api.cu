@@ -93,7 +93,6 @@ void finish_scalars(Scalars* s) {
   s->f_wall_T[1] = (float)s->wall_T[1];
   s->massless = (s->m == 0.0) ? 1 : 0;
   s->iplane = (int)s->plane;
-  s->inv_tau = 1.0 / s->tau;
   s->f_tau = (float)s->tau;
   s->f_tau_coef = (float)s->tau_coef;
   s->f_m = (float)s->m;

@@ -287,7 +287,9 @@ cudaError_t enqueue_chains(rlbm_batch* b, int nsteps, cudaStream_t st) {
     const long long t = h->t;
     const bool have_prev = h->have_prev;
     h->stream = ws;
+    h->sc.plain = 1;                      // (chain.cuh: the chains share the places)
     const int rc = rlbm_step(h, nsteps);
+    h->sc.plain = 0;
     h->stream = own;
     h->cur = cur;
     h->t = t;

@@ -31,6 +31,7 @@
 #include <vector>
 
 #include "../../include/rlbm.h"
+#include "chain.cuh"
 #include "dd.h"
 #include "fxstep.cuh"
 
@@ -245,10 +246,11 @@ __device__ __forceinline__ Cell1 macro1x(const Tab1x<N>& tb, const S (&g)[2 * N]
 
 template <int N>
 __global__ void __launch_bounds__(kThreads) k_step1x(const __grid_constant__ Tab1x<N> tb, const __grid_constant__ Sc s,
-                                                     const double* __restrict__ fin, double* __restrict__ fout,
+                                                     const double* __restrict__ before, double* __restrict__ fout,
                                                      unsigned long long* status) {
   using namespace rlbm;
   constexpr int Q = 2 * N;
+  const double* const fin = chain_begin(before);
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= s.nx) return;
   double g[Q];
@@ -486,9 +488,10 @@ __device__ __forceinline__ void cell1f(const Tab<float>& tb, const Sc& s, const 
 // rather than by loads in flight.
 template <int N, int CPT>
 __global__ void __launch_bounds__(kThreads) k_step1f(const __grid_constant__ Tab<float> tb,
-                                                     const __grid_constant__ Sc s, const float* __restrict__ fin,
+                                                     const __grid_constant__ Sc s, const float* __restrict__ before,
                                                      float* __restrict__ fout, unsigned long long* status) {
   constexpr int Q = 2 * N;
+  const float* const fin = rlbm::chain_begin(before);
   const int x0 = blockIdx.x * (kThreads * CPT) + threadIdx.x;
   float g[CPT][Q];
 #pragma unroll
@@ -708,6 +711,12 @@ void with_tab1x(const rlbm1_handle* h, F&& f) {
 
 dim3 grid1(int nx) { return dim3((nx + kThreads - 1) / kThreads); }
 
+template <int N>
+cudaError_t launch_step1x(const Tab1x<N>& t, const rlbm1_handle* h) {
+  return rlbm::launch_chained(true, k_step1x<N>, grid1(h->sc.nx), dim3(kThreads), 0, h->stream, t, h->sc,
+                              (const double*)h->buf[h->cur], (double*)h->buf[h->cur ^ 1], h->status);
+}
+
 }  // namespace
 
 extern "C" {
@@ -858,22 +867,17 @@ int rlbm1_init(rlbm1_handle* h, const double* n, const double* ux, const double*
 int rlbm1_step(rlbm1_handle* h, int nsteps) {
   if (!h || nsteps < 0) return RLBM_ERR_INVALID_ARG;
   for (int it = 0; it < nsteps; ++it) {
+    cudaError_t e = cudaSuccess;
     if (h->elem == 4) {
       const float* in = (const float*)h->buf[h->cur];
       float* o = (float*)h->buf[h->cur ^ 1];
       const dim3 gr((h->sc.nx + kThreads * kStep1CPT - 1) / (kThreads * kStep1CPT));
-      switch (h->sc.N) {
-        case 2: k_step1f<2, kStep1CPT><<<gr, kThreads, 0, h->stream>>>(*h->tf, h->sc, in, o, h->status); break;
-        case 3: k_step1f<3, kStep1CPT><<<gr, kThreads, 0, h->stream>>>(*h->tf, h->sc, in, o, h->status); break;
-        case 4: k_step1f<4, kStep1CPT><<<gr, kThreads, 0, h->stream>>>(*h->tf, h->sc, in, o, h->status); break;
-        default: k_step1f<5, kStep1CPT><<<gr, kThreads, 0, h->stream>>>(*h->tf, h->sc, in, o, h->status); break;
-      }
-    } else
-      with_tab1x(h, [&](const auto& t) {
-        k_step1x<<<grid1(h->sc.nx), kThreads, 0, h->stream>>>(t, h->sc, (const double*)h->buf[h->cur],
-                                                              (double*)h->buf[h->cur ^ 1], h->status);
-      });
-    const cudaError_t e = cudaGetLastError();
+      auto k = h->sc.N == 2 ? k_step1f<2, kStep1CPT> : h->sc.N == 3 ? k_step1f<3, kStep1CPT>
+             : h->sc.N == 4 ? k_step1f<4, kStep1CPT> : k_step1f<5, kStep1CPT>;
+      e = rlbm::launch_chained(true, k, gr, dim3(kThreads), 0, h->stream, *h->tf, h->sc, in, o, h->status);
+    } else {
+      with_tab1x(h, [&](const auto& t) { e = launch_step1x(t, h); });
+    }
     if (e != cudaSuccess) return cuda_fail1(h, e, "rlbm1_step");
     h->cur ^= 1;
     h->have_prev = true;

@@ -50,7 +50,7 @@ struct Scalars {
   long long plane;
   int boundary;            // 0 periodic, 1 free-flow in x
   int tau_mode;            // 0 const, 1 field, 2 eta/s
-  double tau, inv_tau;     // const tau and its reciprocal
+  double tau;              // const tau
   double tau_coef;         // (eta/s)(d+2) kappa  (tau = tau_coef / T)
   double m;                // rest mass m~
   double n_ref, T_ref;     // reference state (n_ref = 0: no shift)
@@ -72,6 +72,7 @@ struct Scalars {
   float f_tau, f_tau_coef, f_m, f_n_ref, f_T_ref, f_T00_ref, f_Tii_ref;
   float f_PE_hi, f_PE_lo;  // P_ref + eps_ref as a float-float pair (hi + lo)
   int sym_fw;              // orbit-ordered stencil with exactly symmetric H, with a force or walls
+  int plain;               // the step is launched by itself, not as the one before drains (chain.cuh)
 };
 
 // Parity of the px and py exponents of basis monomial k of setup.h

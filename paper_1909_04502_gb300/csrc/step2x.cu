@@ -274,9 +274,11 @@ constexpr size_t shared2x(int K, int mode, int Q) {
 
 template <int K, int MODE, bool MASSLESS>
 __global__ void __launch_bounds__(kThreads2x, K == 9 ? 5 : 4) k_step2x(const __grid_constant__ Tables2x tb,
-                                                                        const __grid_constant__ StepArgs<double> a) {
+                                                                        const __grid_constant__ StepArgs<double> a,
+                                                                        double inv_tau) {
   extern __shared__ int2 columns[];
   const Scalars& s = a.s;
+  const double* const fin = chain_begin(a.fin);
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
   if (x >= s.nx || y >= s.ny) return;
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
@@ -284,7 +286,7 @@ __global__ void __launch_bounds__(kThreads2x, K == 9 ? 5 : 4) k_step2x(const __g
   const Column R{M.s + K * kThreads2x};                // the rates of a quartet
   double* const F = (double*)(R.s + 4 * kThreads2x);   // streamed populations
   const long long si = sidx(s, x, y);
-  const double* __restrict__ base = a.fin + si;
+  const double* __restrict__ base = fin + si;
   double* const ob = a.fout + si;
   const int P = s.iplane;
 
@@ -321,9 +323,9 @@ __global__ void __launch_bounds__(kThreads2x, K == 9 ? 5 : 4) k_step2x(const __g
       sum += v * __uint_as_float((unsigned)(127 + tb.hk[k]) << 23);
     }
     double it;               // 1 / tau
-    if (s.tau_mode == 1) it = 1.0 / a.tau_field[y * s.nx + x];
+    if (s.tau_mode == 1) it = 1.0 / chained(a.tau_field)[y * s.nx + x];
     else if (s.tau_mode == 2) it = c.T / s.tau_coef;
-    else it = s.inv_tau;
+    else it = inv_tau;
     const double o0 = it * c.U0;
     const int xg = above(sum), xo = above(2.f * fabsf(cut_float(o0)));
     ok = ok && xg < 60 && xg > -60;
@@ -520,8 +522,7 @@ cudaError_t launch2x(const Tables2x& tb, const StepArgs<double>& a, cudaStream_t
                                                (int)shared2x(K, MODE, kMaxQ));
     if (e != cudaSuccess) return e;
   }
-  k_step2x<K, MODE, MASSLESS><<<grid, block, bytes, st>>>(tb, a);
-  return cudaGetLastError();
+  return launch_chained(!a.s.plain, k_step2x<K, MODE, MASSLESS>, grid, block, bytes, st, tb, a, 1.0 / a.s.tau);
 }
 
 template <int K, int MODE>

@@ -3,6 +3,7 @@
 // field extraction.  Instantiated per precision / order in step_o2.cu and
 // step_o3.cu.
 #pragma once
+#include "chain.cuh"
 #include "fpconv.cuh"
 #include "fx64.cuh"
 #include "kernels.cuh"
@@ -841,18 +842,20 @@ constexpr int step_threads_per_sm() {
                         : (QT <= 56 ? 512 : 256);
 }
 
-template <typename S, int QT, bool EX, int KT, int MODE, bool SYM, bool MOUT = false, bool FW = false>
+// PLAIN: for launches that are not chained (the batch's concurrent chains).
+template <typename S, int QT, bool EX, int KT, int MODE, bool SYM, bool MOUT = false, bool FW = false, bool PLAIN = false>
 __global__ void __launch_bounds__(kThreads, step_threads_per_sm<S, QT, MODE, SYM, FW>() / kThreads) k_step(const __grid_constant__ Tables<S> tb,
                                                    const __grid_constant__ StepArgs<S> a) {
+  const S* const fin = PLAIN ? a.fin : chain_begin(a.fin);
   const int x = blockIdx.x * kBX + threadIdx.x;
   const int y = blockIdx.y * kBY + threadIdx.y;
   if (x >= a.s.nx || y >= a.s.ny) return;
   if constexpr (MOUT) {
     S g[QT];
-    gather<S, QT, EX, MODE>(tb, a.s, a.fin, sidx(a.s, x, y), g);
-    collide_store<S, QT, EX, KT, SYM, false, true>(tb, a.s, g, a.fout, a.tau_field, a.status, x, y, a.macro);
+    gather<S, QT, EX, MODE>(tb, a.s, fin, sidx(a.s, x, y), g);
+    collide_store<S, QT, EX, KT, SYM, false, true>(tb, a.s, g, a.fout, chained(a.tau_field), a.status, x, y, a.macro);
   } else {
-    cell_update<S, QT, EX, KT, MODE, false, true, SYM, FW>(tb, a.s, a.fin, a.fout, a.tau_field, a.status, x, y);
+    cell_update<S, QT, EX, KT, MODE, false, true, SYM, FW>(tb, a.s, fin, a.fout, PLAIN ? a.tau_field : chained(a.tau_field), a.status, x, y);
   }
 }
 
@@ -935,9 +938,17 @@ inline dim3 block_dim() { return dim3(kBX, kBY); }
 // populations (no per-population bounds test), otherwise Q <= QT at run time.
 template <typename S, int QT, bool EX, int KT, bool SYM = false, bool MOUT = false, bool FW = false>
 cudaError_t launch_step_q(const Tables<S>& tb, const StepArgs<S>& a, int mode, cudaStream_t st) {
-  if (mode == kOnLattice) k_step<S, QT, EX, KT, kOnLattice, SYM, MOUT, FW><<<grid_for(a.s), block_dim(), 0, st>>>(tb, a);
-  else k_step<S, QT, EX, KT, kBilinear, SYM, MOUT, FW><<<grid_for(a.s), block_dim(), 0, st>>>(tb, a);
-  return cudaGetLastError();
+  if constexpr (sizeof(S) == 4 && SYM && KT == 9 && !MOUT && !FW) {
+    if (a.s.plain) {
+      if (mode == kOnLattice) k_step<S, QT, EX, KT, kOnLattice, SYM, MOUT, FW, true><<<grid_for(a.s), block_dim(), 0, st>>>(tb, a);
+      else k_step<S, QT, EX, KT, kBilinear, SYM, MOUT, FW, true><<<grid_for(a.s), block_dim(), 0, st>>>(tb, a);
+      return cudaGetLastError();
+    }
+  }
+  return launch_chained(!a.s.plain,
+                        mode == kOnLattice ? k_step<S, QT, EX, KT, kOnLattice, SYM, MOUT, FW>
+                                           : k_step<S, QT, EX, KT, kBilinear, SYM, MOUT, FW>,
+                        grid_for(a.s), block_dim(), 0, st, tb, a);
 }
 
 template <typename S, int QT, bool EX>

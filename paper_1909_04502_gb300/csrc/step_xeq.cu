@@ -190,12 +190,13 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads) k_step_xeq(const __g
                                                                         const __grid_constant__ StepArgs<float> a) {
   using O = Orbits<QT>;
   const Scalars& s = a.s;
+  const float* const fin = chain_begin(a.fin);
   const int x = blockIdx.x * kBX + threadIdx.x;
   const int y = blockIdx.y * kBY + threadIdx.y;
   if (x >= s.nx || y >= s.ny) return;
   const long long si = sidx(s, x, y);
   float g[QT];
-  gather<float, QT, true, MODE>(tb, s, a.fin, si, g);
+  gather<float, QT, true, MODE>(tb, s, fin, si, g);
   float mm[9];
   moments_sym<float, QT>(tb, g, mm);
   Macro M = landau<float, 0>(s, mm);
@@ -204,7 +205,7 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads) k_step_xeq(const __g
   unphysical_to_reference<float>(s, M);
   ff dM[16];
   eq_moments_xeq(M, xq, dM);
-  const float inv_tau = __fdividef(1.f, local_tau<float>(s, a.tau_field, y * s.nx + x, M));
+  const float inv_tau = __fdividef(1.f, local_tau<float>(s, chained(a.tau_field), y * s.nx + x, M));
   const float kt = M.ok ? inv_tau : 0.f;
   const float U0k = M.fU0 * kt, Uxk = M.fUx * kt, Uyk = M.fUy * kt;
   float* __restrict__ obase = a.fout + si;
@@ -294,9 +295,8 @@ __global__ void __launch_bounds__(kThreads) k_init_xeq(const __grid_constant__ T
 template <int QT>
 cudaError_t launch_xeq_q(const Tables<float>& tb, const XeqTables& xq, const StepArgs<float>& a, int mode,
                          cudaStream_t st) {
-  if (mode == kOnLattice) k_step_xeq<QT, kOnLattice><<<grid_for(a.s), block_dim(), 0, st>>>(tb, xq, a);
-  else k_step_xeq<QT, kBilinear><<<grid_for(a.s), block_dim(), 0, st>>>(tb, xq, a);
-  return cudaGetLastError();
+  return launch_chained(!a.s.plain, mode == kOnLattice ? k_step_xeq<QT, kOnLattice> : k_step_xeq<QT, kBilinear>, grid_for(a.s),
+                        block_dim(), 0, st, tb, xq, a);
 }
 
 }  // namespace
