@@ -639,6 +639,16 @@ int rlbm_step_kernel(const rlbm_handle* h) { return h ? effective_step_kernel(h)
 int rlbm_step(rlbm_handle* h, int nsteps) {
   if (!h || nsteps < 0) return RLBM_ERR_INVALID_ARG;
   const int mode = h->p.stream_mode == RLBM_BILINEAR ? kBilinear : kOnLattice;
+  if (nsteps && h->elem == 4 && h->step_kernel == RLBM_KERNEL_AUTO && row_steps_supported(h->sc)) {
+    StepArgs<float> a{h->sc, (const float*)h->buf[h->cur], (float*)h->buf[h->cur ^ 1],
+                      (const float*)h->tau_field, h->status};
+    const cudaError_t e = launch_row_steps(*h->tf, a, mode, nsteps, h->stream);
+    if (e != cudaSuccess) return cuda_fail(h, e, "step kernel");
+    h->cur ^= nsteps & 1;
+    h->t += nsteps;
+    h->have_prev = true;
+    return RLBM_OK;
+  }
   for (int it = 0; it < nsteps; ++it) {
     cudaError_t e;
     if (h->elem == 4) {

@@ -33,21 +33,35 @@ __device__ __forceinline__ T* chained(T* p) {
 }
 
 template <typename... P, typename... A>
-cudaError_t launch_chained(bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t shared, cudaStream_t st,
-                           const A&... args) {
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
+cudaError_t launch_chained_clusters(bool chained, int cluster, void (*kernel)(P...), dim3 grid, dim3 block, size_t shared,
+                                    cudaStream_t st, const A&... args) {
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (chained) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = (unsigned)cluster;
+    attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
+    ++n;
+  }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = shared;
   cfg.stream = st;
-  cfg.attrs = &attr;
-  cfg.numAttrs = chained ? 1 : 0;
+  cfg.attrs = attr;
+  cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+template <typename... P, typename... A>
+cudaError_t launch_chained(bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t shared, cudaStream_t st,
+                           const A&... args) {
+  return launch_chained_clusters(chained, 1, kernel, grid, block, shared, st, args...);
+}
 #endif
 
 }  // namespace rlbm

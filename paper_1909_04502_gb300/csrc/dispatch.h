@@ -31,6 +31,13 @@ cudaError_t launch_step_xeq(const Tables<float>& tb, const XeqTables& xq, const 
 cudaError_t launch_init_xeq(const Tables<float>& tb, const XeqTables& xq, const InitArgs<float>& a,
                             cudaStream_t st);
 
+// One-row grids (step_row.cu): nsteps steps from a.fin, between a.fin and
+// a.fout, with the images of both; the images along y of the row of f.
+bool row_steps_supported(const Scalars& s);
+cudaError_t launch_row_steps(const Tables<float>& tb, const StepArgs<float>& a, int mode, int nsteps, cudaStream_t st);
+template <typename S>
+cudaError_t launch_row_images(S* f, const Scalars& s, cudaStream_t st);
+
 template <typename S>
 inline cudaError_t launch_step(const Tables<S>& tb, const StepArgs<S>& a, int mode, cudaStream_t st) {
   return a.s.K == 9 ? launch_step_k9<S>(tb, a, mode, st) : launch_step_k16<S>(tb, a, mode, st);

@@ -94,6 +94,14 @@ __host__ __device__ __forceinline__ long long sidx(const Scalars& s, int x, int 
   return (long long)(y + s.hy) * s.pitch + (x + s.px);
 }
 
+// The row of a one-row grid by itself: no images along y, and every y offset
+// of a pull falls on it (the buffers then start at row hy of the storage).
+inline Scalars row_scalars(Scalars s) {
+  s.hy = 0;
+  s.pitch = 0;
+  return s;
+}
+
 // Macroscopic state of f(t+1)'s cells as the FP32-storage step leaves it:
 // planes n, T, U^0, U^x, U^y, n - n_ref, T - T_ref, eps ([kMacroPlanes][ncell]).
 constexpr int kMacroPlanes = 8;

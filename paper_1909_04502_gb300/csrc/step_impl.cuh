@@ -4,6 +4,7 @@
 // step_o3.cu.
 #pragma once
 #include "chain.cuh"
+#include "dispatch.h"
 #include "fpconv.cuh"
 #include "fx64.cuh"
 #include "kernels.cuh"
@@ -903,24 +904,27 @@ __global__ void __launch_bounds__(kThreads) k_fields(const __grid_constant__ Tab
 }
 
 // Initialisation f*(0) = f^eq(n, U, T) (Sec. 6.2), stored shifted, with halo images.
-template <typename S, int KT>
-__global__ void __launch_bounds__(kThreads) k_init(const __grid_constant__ Tables<S> tb,
+constexpr int kInitWarps = 16;
+// ROW: a grid of one row without its images along y (launch_row_images), the
+// populations shared out over the warps (1024 cells: 129 -> 10 us).
+template <typename S, int KT, bool ROW>
+__global__ void __launch_bounds__(ROW ? 32 * kInitWarps : kThreads) k_init(const __grid_constant__ Tables<S> tb,
                                                    const __grid_constant__ InitArgs<S> a) {
   const int x = blockIdx.x * kBX + threadIdx.x;
-  const int y = blockIdx.y * kBY + threadIdx.y;
+  const int y = ROW ? 0 : blockIdx.y * kBY + threadIdx.y;
   if (x >= a.s.nx || y >= a.s.ny) return;
   const int cell = y * a.s.nx + x;
   const double ux = a.ux[cell], uy = a.uy[cell];
   const double u2 = ux * ux + uy * uy;
   const double n = a.n[cell], T = a.T[cell];
   const bool ok = (u2 < 1.0) && (n > 0.0) && (T > 0.0);
-  if (!ok) atomicAdd(a.status, 1ULL);
+  if (!ok && (!ROW || threadIdx.y == 0)) atomicAdd(a.status, 1ULL);
   const double gam = ok ? 1.0 / sqrt(1.0 - u2) : 1.0;
   S dM[KT];
   eq_moments<S, KT>((S)(n - a.s.n_ref), (S)(T - a.s.T_ref), (S)n, (S)T, (S)gam, (S)(gam * ux),
                     (S)(gam * uy), (S)a.s.m, (S)a.s.n_ref, (S)a.s.T_ref, dM);
   const long long si = sidx(a.s, x, y);
-  for (int i = 0; i < a.s.Q; ++i) {
+  for (int i = ROW ? threadIdx.y : 0; i < a.s.Q; i += ROW ? kInitWarps : 1) {
     S feq = S(0);
 #pragma unroll
     for (int k = 0; k < KT; ++k) feq = fma(tb.H[i][k], dM[k], feq);
@@ -960,7 +964,15 @@ cudaError_t launch_fields_q(const Tables<S>& tb, const MomentArgs<S>& a, int mod
 
 template <typename S, int KT>
 cudaError_t launch_init_k(const Tables<S>& tb, const InitArgs<S>& a, cudaStream_t st) {
-  k_init<S, KT><<<grid_for(a.s), block_dim(), 0, st>>>(tb, a);
+  if (a.s.ny == 1) {
+    InitArgs<S> r = a;
+    r.s = row_scalars(a.s);
+    r.fout += (long long)a.s.hy * a.s.pitch;
+    k_init<S, KT, true><<<(a.s.nx + 31) / 32, dim3(32, kInitWarps), 0, st>>>(tb, r);
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e : launch_row_images<S>(a.fout, a.s, st);
+  }
+  k_init<S, KT, false><<<grid_for(a.s), block_dim(), 0, st>>>(tb, a);
   return cudaGetLastError();
 }
 
