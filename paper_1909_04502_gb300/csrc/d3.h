@@ -27,6 +27,7 @@ struct Scalars3 {
   double tau, inv_tau;
   double n_ref, T_ref;    // FP32 storage reference state (0, 0 for FP64 storage)
   float f_n_ref, f_T_ref, f_inv_tau;   // FP32 copies of n_ref, T_ref and 1 / tau
+  float f_e_ref, f_P_ref;              // and of the reference state's energy density and pressure
 };
 
 // S: storage type (double: f; float: g = f - f_ref)

@@ -23,33 +23,6 @@ __device__ __forceinline__ int images1(int c, int n, int h, int (&out)[2]) {
   return k;
 }
 
-template <typename R>
-__device__ __forceinline__ R det3(R a, R b, R c, R d, R e, R f, R g, R hh, R i) {
-  return a * (e * i - f * hh) - b * (d * i - f * g) + c * (d * hh - e * g);
-}
-
-// det(B) by complementary 2 x 2 minors of rows (0, 1) and (2, 3), and
-// d det(B - l I)/dl = -(sum of the principal 3 x 3 minors)
-template <typename R>
-__device__ __forceinline__ R det4(const R (&B)[4][4]) {
-  const R s0 = B[0][0] * B[1][1] - B[1][0] * B[0][1], s1 = B[0][0] * B[1][2] - B[1][0] * B[0][2];
-  const R s2 = B[0][0] * B[1][3] - B[1][0] * B[0][3], s3 = B[0][1] * B[1][2] - B[1][1] * B[0][2];
-  const R s4 = B[0][1] * B[1][3] - B[1][1] * B[0][3], s5 = B[0][2] * B[1][3] - B[1][2] * B[0][3];
-  const R c5 = B[2][2] * B[3][3] - B[3][2] * B[2][3], c4 = B[2][1] * B[3][3] - B[3][1] * B[2][3];
-  const R c3 = B[2][1] * B[3][2] - B[3][1] * B[2][2], c2 = B[2][0] * B[3][3] - B[3][0] * B[2][3];
-  const R c1 = B[2][0] * B[3][2] - B[3][0] * B[2][2], c0 = B[2][0] * B[3][1] - B[3][0] * B[2][1];
-  return s0 * c5 - s1 * c4 + s2 * c3 + s3 * c2 - s4 * c1 + s5 * c0;
-}
-
-template <typename R>
-__device__ __forceinline__ R ddet4(const R (&B)[4][4]) {
-  const R m0 = det3(B[1][1], B[1][2], B[1][3], B[2][1], B[2][2], B[2][3], B[3][1], B[3][2], B[3][3]);
-  const R m1 = det3(B[0][0], B[0][2], B[0][3], B[2][0], B[2][2], B[2][3], B[3][0], B[3][2], B[3][3]);
-  const R m2 = det3(B[0][0], B[0][1], B[0][3], B[1][0], B[1][1], B[1][3], B[3][0], B[3][1], B[3][3]);
-  const R m3 = det3(B[0][0], B[0][1], B[0][2], B[1][0], B[1][1], B[1][2], B[2][0], B[2][1], B[2][2]);
-  return -(m0 + m1 + m2 + m3);
-}
-
 // right null vector of B from the first column of adj(B):
 // v_i = (-1)^i det(B without row 0 and column i), each 3 x 3 minor expanded
 // along row 1 over the six 2 x 2 minors c_ab of rows 2 and 3; B v = det(B) e_0,
@@ -115,82 +88,87 @@ struct Macro3f {
 
 __device__ __forceinline__ Macro3f landau3f(const float (&N)[4], const float (&Tm)[4][4], const Scalars3& s) {
   const double nr = s.n_ref, Tr = s.T_ref, er = 3.0 * nr * Tr, Pr = nr * Tr;
-  const float fnr = d2f(nr), fTr = d2f(Tr), fer = d2f(er), fPr = d2f(Pr);
-  // the mixed tensor A = T eta in FP32 (reference diagonal added)
-  float Af[4][4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      float t = u <= v ? Tm[u][v] : Tm[v][u];
-      if (u == v) t += (u == 0 ? fer : fPr);
-      Af[u][v] = v == 0 ? t : -t;
-    }
+  const float fnr = s.f_n_ref, fTr = s.f_T_ref;
+  // T^ab = (E, s; s, P) in FP32 (reference diagonal added); the mixed tensor
+  // A = T eta has det(A - l I) = (l - E) D(l) + S(l), D = det(P + l I) =
+  // l^3 + a1 l^2 + a2 l + a3, S = s . adj(P + l I) s = b0 l^2 + b1 l + b2
+  const float E = Tm[0][0] + s.f_e_ref, x = Tm[0][1], y = Tm[0][2], z = Tm[0][3];
+  const float pxx = Tm[1][1] + s.f_P_ref, pyy = Tm[2][2] + s.f_P_ref, pzz = Tm[3][3] + s.f_P_ref;
+  const float pxy = Tm[1][2], pxz = Tm[1][3], pyz = Tm[2][3];
+  const float cxx = pyy * pzz - pyz * pyz, cyy = pxx * pzz - pxz * pxz, czz = pxx * pyy - pxy * pxy;
+  const float cxy = pxz * pyz - pxy * pzz, cxz = pxy * pyz - pxz * pyy, cyz = pxy * pxz - pyz * pxx;
+  const float a1 = pxx + pyy + pzz, a2 = cxx + cyy + czz, a3 = pxx * cxx + pxy * cxy + pxz * cxz;
+  const float xx = x * x, yy = y * y, zz = z * z, xy = 2.f * x * y, xz = 2.f * x * z, yz = 2.f * y * z;
+  const float b0 = xx + yy + zz;
+  const float b1 = a1 * b0 - (xx * pxx + yy * pyy + zz * pzz + xy * pxy + xz * pxz + yz * pyz);
+  const float b2 = xx * cxx + yy * cyy + zz * czz + xy * cxy + xz * cxz + yz * cyz;
   // FP32 root from the ideal-fluid guess (P = eps / 3)
-  const float E = Af[0][0], M2 = Af[1][0] * Af[1][0] + Af[2][0] * Af[2][0] + Af[3][0] * Af[3][0];
   const float k = 1.f / 3.f;
-  float lam = (-(1.f - k) * E + sqrtf(fmaxf((1.f - k) * (1.f - k) * E * E + 4.f * k * (E * E - M2), 0.f))) /
-              (2.f * k);
-  float Bf[4][4];
+  float lam = (-(1.f - k) * E + sqrtf(fmaxf((1.f - k) * (1.f - k) * E * E + 4.f * k * (E * E - b0), 0.f))) * 1.5f;
   float dpf = -1.f;
 #pragma unroll
   for (int it = 0; it < 3; ++it) {
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-      for (int v = 0; v < 4; ++v) Bf[u][v] = Af[u][v] - (u == v ? lam : 0.f);
-    dpf = ddet4(Bf);
-    lam -= det4(Bf) / dpf;
+    const float D = fmaf(fmaf(lam + a1, lam, a2), lam, a3), dD = fmaf(fmaf(3.f, lam, 2.f * a1), lam, a2);
+    const float S = fmaf(fmaf(b0, lam, b1), lam, b2), dS = fmaf(2.f * b0, lam, b1);
+    dpf = fmaf(lam - E, dD, D + dS);
+    lam -= __fdividef(fmaf(lam - E, D, S), dpf);
   }
   // FP64 residual at the FP32 root: B = A - l I with A's entries exact from
   // the FP32 sums and the FP64 reference
-  const double ld = f2d(lam);
+  const double ld = f2d_finite(lam);
   const double d0 = ld - er, d1 = Pr + ld;
   double B[4][4];
 #pragma unroll
   for (int u = 0; u < 4; ++u)
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
-      const double t = f2d(u <= v ? Tm[u][v] : Tm[v][u]);
+      const double t = f2d_finite(u <= v ? Tm[u][v] : Tm[v][u]);
       B[u][v] = v == 0 ? t : -t;
     }
-  B[0][0] = f2d(Tm[0][0]) - d0;
+  B[0][0] = f2d_finite(Tm[0][0]) - d0;
 #pragma unroll
-  for (int u = 1; u < 4; ++u) B[u][u] = -(f2d(Tm[u][u]) + d1);
+  for (int u = 1; u < 4; ++u) B[u][u] = -(f2d_finite(Tm[u][u]) + d1);
   double vv[4];
   adj_col0(B, vv);
+  int top = 0;
   const double p = B[0][0] * vv[0] + B[0][1] * vv[1] + B[0][2] * vv[2] + B[0][3] * vv[3];
-  const float dl = -__fdividef(d2f(p), dpf);
+  const float dl = -__fdividef(d2f_finite(p, top), dpf);
   // the eigenvector at l + dl to first order
-#pragma unroll
-  for (int u = 0; u < 4; ++u) Bf[u][u] = Af[u][u] - lam;
+  const float Bf[4][4] = {{E - lam, -x, -y, -z},
+                          {x, -(pxx + lam), -pxy, -pxz},
+                          {y, -pxy, -(pyy + lam), -pyz},
+                          {z, -pxz, -pyz, -(pzz + lam)}};
   float dv[4];
   dadj_col0(Bf, dv);
   double vc[4];
 #pragma unroll
-  for (int u = 0; u < 4; ++u) vc[u] = vv[u] + f2d(dl * dv[u]);
+  for (int u = 0; u < 4; ++u) vc[u] = vv[u] + f2d_finite(dl * dv[u]);
   const double nu2 = vc[0] * vc[0] - vc[1] * vc[1] - vc[2] * vc[2] - vc[3] * vc[3];
-  const double w = vc[0] * (nr + f2d(N[0])) - vc[1] * f2d(N[1]) - vc[2] * f2d(N[2]) - vc[3] * f2d(N[3]);
+  const double w = vc[0] * (nr + f2d_finite(N[0])) - vc[1] * f2d_finite(N[1]) - vc[2] * f2d_finite(N[2]) -
+                   vc[3] * f2d_finite(N[3]);
   const double num = fma(w, w, -(nr * nr) * nu2);
-  const double deps = d0 + f2d(dl);
+  const double deps = d0 + f2d_finite(dl);
   // FP32 quotients
-  const float fnu2 = d2f(nu2);
+  const float fnu2 = d2f_finite(nu2, top);
   const float inu = rsqrtf(fnu2);
   const float fnu = fnu2 * inu;
   const float sgn = __double2hiint(vc[0]) < 0 ? -1.f : 1.f;
-  const float fw = sgn * d2f(w);
+  const float fw = sgn * d2f_finite(w, top);
   Macro3f M;
   M.n = fw * inu;
-  M.dn = __fdividef(d2f(num), fnu * (fw + fnr * fnu));
-  M.dT = __fdividef(d2f(deps) - 3.f * fTr * M.dn, 3.f * M.n);
+  M.dn = __fdividef(d2f_finite(num, top), fnu * (fw + fnr * fnu));
+  M.dT = __fdividef(d2f_finite(deps, top) - 3.f * fTr * M.dn, 3.f * M.n);
   M.T = fTr + M.dT;
   const float su = sgn * inu;
-  M.U0 = d2f(vc[0]) * su;
-  M.Ux = d2f(vc[1]) * su;
-  M.Uy = d2f(vc[2]) * su;
-  M.Uz = d2f(vc[3]) * su;
+  M.U0 = d2f_finite(vc[0], top) * su;
+  M.Ux = d2f_finite(vc[1], top) * su;
+  M.Uy = d2f_finite(vc[2], top) * su;
+  M.Uz = d2f_finite(vc[3], top) * su;
+  // the conversions take finite values: lam and dl are not finite when a T^ab
+  // or the frame is not, and the FP64 values are checked by their magnitude
   M.ok = (__double2hiint(nu2) > 0) && (M.n > 0.f) && (M.T > 0.f) && isfinite(M.T) && isfinite(M.dn) &&
-         isfinite(M.n);
+         isfinite(M.n) && isfinite(lam) && isfinite(dl * (dv[0] + dv[1] + dv[2] + dv[3])) &&
+         isfinite(N[0] + N[1] + N[2] + N[3]) && top < kNoFloat;
   return M;
 }
 
@@ -227,6 +205,11 @@ __device__ __forceinline__ void mj_full3(double n, double T, const double (&U)[4
   }
 }
 
+__device__ __forceinline__ float quotient32(float a, float b) {     // b normal and below 2^126
+  const float r = __fdividef(1.f, b), q = a * r;
+  return fmaf(fmaf(-b, q, a), r, q);
+}
+
 // Differences dM = M(n, U, T) - M(n_ref, rest, T_ref) (FP32 storage), each
 // written so that it is accurate relative to itself given accurate dn, dT:
 //   <1>: (dn T_ref - n_ref dT) / (2 T T_ref);  <p0>: dn U0 + n_ref (U0 - 1);
@@ -237,9 +220,9 @@ template <int K>
 __device__ __forceinline__ void mj_delta3(const Macro3f& M, float nr, float Tr, float (&dM)[K]) {
   const float U[4] = {M.U0, M.Ux, M.Uy, M.Uz};
   const float n = M.n, T = M.T, dn = M.dn, dT = M.dT;
-  const float U0m1 = (M.Ux * M.Ux + M.Uy * M.Uy + M.Uz * M.Uz) / (M.U0 + 1.f);
+  const float U0m1 = quotient32(M.Ux * M.Ux + M.Uy * M.Uy + M.Uz * M.Uz, M.U0 + 1.f);
   const float q = 4.f * n * T, iso = dn * T + nr * dT;
-  dM[0] = (dn * Tr - nr * dT) / (2.f * T * Tr);
+  dM[0] = quotient32(dn * Tr - nr * dT, 2.f * T * Tr);
   dM[1] = dn * M.U0 + nr * U0m1;
   dM[2] = n * M.Ux;
   dM[3] = n * M.Uy;

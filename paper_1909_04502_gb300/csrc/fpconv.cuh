@@ -41,6 +41,28 @@ __device__ __forceinline__ float d2f(double d) {
   return __uint_as_float(b);
 }
 
+// The same without the special classes, in half the operations.  f2d_finite:
+// a finite float; zero and denormals become a value below 2^-126 instead of zero.
+// d2f_finite: rounds as d2f does; a magnitude below 2^-126 becomes one below 2^-125,
+// and `top` collects the largest magnitude's high word, by which the caller
+// tells values that no float holds (top >= kNoFloat: 2^127 and above,
+// infinities, NaNs).
+constexpr int kNoFloat = 0x47E00000;
+
+__device__ __forceinline__ double f2d_finite(float f) {
+  const unsigned b = __float_as_uint(f);
+  return __hiloint2double((int)((((b & 0x7FFFFFFFu) >> 3) + 0x38000000u) | (b & 0x80000000u)), (int)(b << 29));
+}
+
+__device__ __forceinline__ float d2f_finite(double d, int& top) {
+  const unsigned lo = (unsigned)__double2loint(d), lo2 = lo + (1u << 28);
+  const int hw = __double2hiint(d);
+  const int hi = (hw & 0x7FFFFFFF) + (lo2 < lo ? 1 : 0);
+  top = max(top, hi);
+  const unsigned b = __funnelshift_l(lo2, (unsigned)(max(hi, 0x38100000) - 0x38000000), 3);
+  return __uint_as_float(b | ((unsigned)hw & 0x80000000u));
+}
+
 // Float-float arithmetic: a value is the unevaluated sum hi + lo of two FP32
 // numbers (about 48 significant bits), built on error-free transformations
 // (Knuth's two-sum, the FMA two-product).  It runs on the FP32 pipe, whose

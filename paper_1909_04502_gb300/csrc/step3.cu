@@ -24,6 +24,18 @@ __device__ constexpr int kBasis3Exp[14][3] = {{0, 0, 0}, {0, 0, 0}, {1, 0, 0}, {
                                               {1, 0, 0}, {0, 1, 0}, {0, 0, 1}, {2, 0, 0}, {1, 1, 0},
                                               {1, 0, 1}, {0, 2, 0}, {0, 1, 1}, {0, 0, 2}};
 
+__device__ __forceinline__ void copy_async4(float* to, const void* from) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(to)), "l"(from) : "memory");
+}
+// all but the newest n groups have arrived
+__device__ __forceinline__ void wait_copies(int n) {
+  switch (n) {
+#define WAIT(k) case k: asm volatile("cp.async.wait_group " #k ";" ::: "memory"); break;
+    WAIT(0) WAIT(1) WAIT(2) WAIT(3) WAIT(4) WAIT(5) WAIT(6) WAIT(7) WAIT(8) WAIT(9)
+#undef WAIT
+  }
+}
+
 // The FP32-storage step in sign-orbit form.
 // Populations come in runs whose members share p0 and |p| componentwise:
 // 9 runs of 8 (member s negates the components whose bit is set in s) and
@@ -47,17 +59,32 @@ __device__ constexpr int kBasis3Exp[14][3] = {{0, 0, 0}, {0, 0, 0}, {1, 0, 0}, {
 // FP32.  Every run is unrolled, so each table entry (pull shift, monomial, H
 // row, velocity) is an immediate constant operand rather than a load by
 // run-time index (with the runs in a loop this form was slower than the
-// row-by-row kernel it replaced).  Eight blocks of 128 threads per SM
-// (64 registers).  At 192^3: 1.51 ms per step against 2.20 ms row by row.
-// The interior is stored in the relaxation pass; cells next to a face then
-// copy their values to the periodic images, six at a time.
+// row-by-row kernel it replaced).
+// The pulled populations go to shared memory by asynchronous copies, all 78 in
+// flight at once, and both passes read them there (40 KB per block of 128
+// threads, five blocks per SM); the relaxed values stay there for the periodic
+// images of the cells next to a face.  At 192^3: 1.37 ms per step (0.48 of the
+// copy bandwidth), at 96^3 217 us, at 33^3 25 us, against 1.50 ms, 262 us and
+// 44 us with the populations pulled again in the second pass by eight blocks per SM,
+// the images copied from the stored values and the former frame3.  What bounds
+// it: about 2870 instructions per cell at 5 warps per scheduler, whose phases
+// (copies, FP64 frame, stores) overlap in part; without the images 1.28 ms.
+// Half of the populations kept and eight blocks per SM: 1.48 ms.
 __global__ void __launch_bounds__(128, 8) k_step3fs(const __grid_constant__ Tables3 tb,
                                                     const __grid_constant__ Step3Args<float> a) {
   const Scalars3& s = a.s;
   const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 4 + threadIdx.y, z = blockIdx.z;
   if (x >= s.nx || y >= s.ny || z >= s.nz) return;
-  const long long si = sidx3(s, x, y, z);
-  const float* __restrict__ base = a.fin + si;
+  // (addresses: a plane's uniform one plus the cell's 32-bit offset)
+  const unsigned cell = (unsigned)sidx3(s, x, y, z) * 4u;
+  // the pulled populations, a column per thread: a group of copies per run
+  __shared__ float columns[78 * 128];
+  float* F = columns + threadIdx.y * 32 + threadIdx.x;
+#pragma unroll
+  for (int i = 0; i < 78; ++i) {
+    copy_async4(F + i * 128, (const char*)(a.fin + tb.off[i]) + cell);
+    if (i % 8 == 7 || i == 77) asm volatile("cp.async.commit_group;" ::: "memory");
+  }
   // pass 1: m = N0 Nx Ny Nz T00 T0x T0y T0z Txx Txy Txz Tyy Tyz Tzz of g
   float m[14];
 #pragma unroll
@@ -65,14 +92,16 @@ __global__ void __launch_bounds__(128, 8) k_step3fs(const __grid_constant__ Tabl
 #pragma unroll
   for (int r = 0; r < 9; ++r) {
     float f[8];
+    wait_copies(9 - r);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) f[q] = __ldg(base + tb.off[8 * r + q]);
+    for (int q = 0; q < 8; ++q) f[q] = F[(8 * r + q) * 128];
     fwht(f);
     moments_run8(f, tb.monof[r], m);
   }
+  wait_copies(0);
 #pragma unroll
   for (int ax = 0; ax < 3; ++ax) {
-    const float fp = __ldg(base + tb.off[72 + 2 * ax]), fm = __ldg(base + tb.off[73 + 2 * ax]);
+    const float fp = F[(72 + 2 * ax) * 128], fm = F[(73 + 2 * ax) * 128];
     const float Sm = fp + fm, D = fp - fm;
     const float* c = tb.monof[9 + ax];
     const int taa = ax == 0 ? 8 : (ax == 1 ? 11 : 13);
@@ -86,8 +115,12 @@ __global__ void __launch_bounds__(128, 8) k_step3fs(const __grid_constant__ Tabl
   if (!frame3(m, s, Mm, kU0, kU)) atomicAdd(a.status, 1ULL);
   // pass 2: equilibrium differences, relaxation, interior store (order 2
   // keeps Q * plane below 2^31)
-  const int ipl = (int)s.plane;
-  float* ob = a.fout + si;
+  int tx, ty;                          // (read again: no registers held for them meanwhile)
+  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tx));
+  asm volatile("mov.u32 %0, %%tid.y;" : "=r"(ty));
+  const unsigned to = (unsigned)sidx3(s, blockIdx.x * 32 + tx, blockIdx.y * 4 + ty, blockIdx.z) * 4u;
+  auto plane = [&](int i) { return (char*)(a.fout + (long long)i * s.plane); };
+  F = columns + ty * 32 + tx;
 #pragma unroll
   for (int r = 0; r < 9; ++r) {
     const float* H0 = tb.Hf[8 * r];
@@ -109,8 +142,8 @@ __global__ void __launch_bounds__(128, 8) k_step3fs(const __grid_constant__ Tabl
     for (int q = 0; q < 8; ++q) {
       const int i = 8 * r + q;
       const float om = (q & 4) ? R[q & 3] + Z : R[q & 3] - Z;
-      const float g = __ldg(base + tb.off[i]);
-      ob[i * ipl] = fmaf(om, C[q] - g, g);
+      const float g = F[i * 128];
+      *(float*)(plane(i) + to) = F[i * 128] = fmaf(om, C[q] - g, g);
     }
   }
 #pragma unroll
@@ -129,11 +162,17 @@ __global__ void __launch_bounds__(128, 8) k_step3fs(const __grid_constant__ Tabl
       const int i = i0 + q;
       const float feq = q ? Ce - Co : Ce + Co;
       const float om = q ? kU0 + va : kU0 - va;
-      const float g = __ldg(base + tb.off[i]);
-      ob[i * ipl] = fmaf(om, feq - g, g);
+      const float g = F[i * 128];
+      *(float*)(plane(i) + to) = F[i * 128] = fmaf(om, feq - g, g);
     }
   }
-  images_from_stored<78, 6>(s, a.fout, si, x, y, z);
+  long long img[26];
+  const int images = cell_images(s, blockIdx.x * 32 + tx, blockIdx.y * 4 + ty, blockIdx.z, img);
+  for (int k = 0; k < images; ++k) {
+    const unsigned at = (unsigned)img[k] * 4u;
+#pragma unroll 6
+    for (int i = 0; i < 78; ++i) *(float*)(plane(i) + at) = F[i * 128];
+  }
 }
 
 // f*(0) = f^eq(n, U, T) of device fields (row-major [z][y][x]), stored as f
