@@ -166,7 +166,7 @@ __device__ __forceinline__ Macro3f landau3f(const float (&N)[4], const float (&T
   M.Uz = d2f_finite(vc[3], top) * su;
   // the conversions take finite values: lam and dl are not finite when a T^ab
   // or the frame is not, and the FP64 values are checked by their magnitude
-  M.ok = (__double2hiint(nu2) > 0) && (M.n > 0.f) && (M.T > 0.f) && isfinite(M.T) && isfinite(M.dn) &&
+  M.ok = (__double2hiint(nu2) >= kLeastFloat) && (M.n > 0.f) && (M.T > 0.f) && isfinite(M.T) && isfinite(M.dn) &&
          isfinite(M.n) && isfinite(lam) && isfinite(dl * (dv[0] + dv[1] + dv[2] + dv[3])) &&
          isfinite(N[0] + N[1] + N[2] + N[3]) && top < kNoFloat;
   return M;

@@ -43,11 +43,11 @@ __device__ __forceinline__ float d2f(double d) {
 
 // The same without the special classes, in half the operations.  f2d_finite:
 // a finite float; zero and denormals become a value below 2^-126 instead of zero.
-// d2f_finite: rounds as d2f does; a magnitude below 2^-126 becomes one below 2^-125,
-// and `top` collects the largest magnitude's high word, by which the caller
+// d2f_finite: rounds as d2f does; a magnitude below 2^-120 becomes zero (with it
+// what f2d_finite made of zeros), and `top` collects the largest magnitude's high word, by which the caller
 // tells values that no float holds (top >= kNoFloat: 2^127 and above,
 // infinities, NaNs).
-constexpr int kNoFloat = 0x47E00000;
+constexpr int kNoFloat = 0x47E00000, kLeastFloat = 0x38700000;
 
 __device__ __forceinline__ double f2d_finite(float f) {
   const unsigned b = __float_as_uint(f);
@@ -59,8 +59,8 @@ __device__ __forceinline__ float d2f_finite(double d, int& top) {
   const int hw = __double2hiint(d);
   const int hi = (hw & 0x7FFFFFFF) + (lo2 < lo ? 1 : 0);
   top = max(top, hi);
-  const unsigned b = __funnelshift_l(lo2, (unsigned)(max(hi, 0x38100000) - 0x38000000), 3);
-  return __uint_as_float(b | ((unsigned)hw & 0x80000000u));
+  const unsigned b = __funnelshift_l(lo2, (unsigned)(hi - 0x38000000), 3) | ((unsigned)hw & 0x80000000u);
+  return __uint_as_float(hi >= kLeastFloat ? b : 0u);
 }
 
 // Float-float arithmetic: a value is the unevaluated sum hi + lo of two FP32
