@@ -15,7 +15,7 @@
 // What bounds it: integer issue at 20 warps per SM (about 180 instructions per
 // population and step; the sums in FP64 held that pipe at 85 % and took 540 to
 // 980 operations per cell of it, 80 to 160 are left).  517 x 333, massless order 2:
-// 62 us per step and 18 us for the fields against 190 and 139 us; 512 x 512,
+// 56 us per step (chained) and 18 us for the fields against 190 and 139 us; 512 x 512,
 // m = 5, order 3 (49 populations): 160 and 40 us against 445 and 300 us.
 #include <cuda_runtime.h>
 

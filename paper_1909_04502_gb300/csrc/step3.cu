@@ -63,7 +63,7 @@ __device__ __forceinline__ void wait_copies(int n) {
 // The pulled populations go to shared memory by asynchronous copies, all 78 in
 // flight at once, and both passes read them there (40 KB per block of 128
 // threads, five blocks per SM); the relaxed values stay there for the periodic
-// images of the cells next to a face.  At 192^3: 1.37 ms per step (0.48 of the
+// images of the cells next to a face.  At 192^3: 1.39 ms per step (0.47 of the
 // copy bandwidth), at 96^3 217 us, at 33^3 25 us, against 1.50 ms, 262 us and
 // 44 us with the populations pulled again in the second pass by eight blocks per SM,
 // the images copied from the stored values and the former frame3.  What bounds
