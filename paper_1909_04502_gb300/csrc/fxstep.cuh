@@ -1,5 +1,6 @@
 // Device helpers shared by the fixed-point steps (step2x.cu, step3x.cu).
 #pragma once
+#include "frame64.cuh"
 #include "fx64.cuh"
 
 namespace rlbm {
@@ -69,6 +70,23 @@ __device__ __forceinline__ double scaled(double v, int k) {
   if (__builtin_expect(e > 0 && e < 0x7FF && e + k > 0 && e + k < 0x7FF, 1))
     return __hiloint2double(h + (k << 20), __double2loint(v));
   return scaled_any(v, k);
+}
+
+// 2^lo <= v < 2^hi (false for NaN)
+__device__ __forceinline__ bool between(double v, int lo, int hi) {
+  return (unsigned)(__double2hiint(v) - ((1023 + lo) << 20)) < (unsigned)((hi - lo) << 20);
+}
+
+// frame64 out of line: v = T00, T0i, Txx Txy Txz Tyy Tyz Tzz becomes l, u; in
+// memory, so that the caller holds no registers for them.
+__device__ __noinline__ bool settle_frame(double* v) {
+  const double t[3] = {v[1], v[2], v[3]}, S[6] = {v[4], v[5], v[6], v[7], v[8], v[9]};
+  const Frame64 f = frame64(v[0], t, S);
+  v[0] = f.l;
+  v[1] = f.u[0];
+  v[2] = f.u[1];
+  v[3] = f.u[2];
+  return f.ok;
 }
 
 // Values of a thread split for products (split_balanced), in a shared-memory

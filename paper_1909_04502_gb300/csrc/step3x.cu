@@ -100,15 +100,16 @@ __device__ __forceinline__ void run_units(const float (&g)[L], int ep, long long
 // u = U^i / U^0 and (T^ij + eps delta^ij) u_j = T^0i, eps = T^00 - T^0i u_i.
 struct Cell3 {
   double L, u[3], U0, n;
-  float fL, fn;              // their leading parts
   bool ok;
 };
 
 // (t = T^0i; S = Txx Txy Txz Tyy Tyz Tzz.)  The root and u in FP32 by Newton on
 // g(l) = T00 - t.(S + l)^-1 t - l, g' = u.u - 1; then (l, u) together by
 // iterative refinement: FP64 residuals of both equations, the correction
-// through the FP32 inverse.  A pass gains about 20 bits; two are enough
-// (a third runs where the second still moved the root by 2^-40).
+// through the FP32 inverse.  A pass gains about 20 bits in slow flows; two are enough
+// (more run where the last still moved l by 2^-40 or u by 2^-36 of 1 - u.u).  The inverse's error
+// grows as gamma^4: what has not settled after six passes is solved in FP64
+// (frame64.cuh; from gamma of about 7 on).
 __device__ __forceinline__ Cell3 landau3x(const double (&N)[4], double T00, const double (&t)[3],
                                           const double (&S)[6]) {
   const float fT = cut_float(T00), ft[3] = {cut_float(t[0]), cut_float(t[1]), cut_float(t[2])};
@@ -146,6 +147,7 @@ __device__ __forceinline__ Cell3 landau3x(const double (&N)[4], double T00, cons
   c.u[1] = wide_double(v[1]);
   c.u[2] = wide_double(v[2]);
   const float iw = __fdividef(1.f, w);
+  bool settled = false;
 #pragma unroll 1
   for (int it = 0; it < 6; ++it) {
     const double r0 = fma(-t[2], c.u[2], fma(-t[1], c.u[1], fma(-t[0], c.u[0], T00 - c.L)));
@@ -155,19 +157,28 @@ __device__ __forceinline__ Cell3 landau3x(const double (&N)[4], double T00, cons
     const float x = cut_float(rx), y = cut_float(ry), z = cut_float(rz);
     const float d = (cut_float(r0) - v[0] * x - v[1] * y - v[2] * z) * iw;
     const float ex = x - v[0] * d, ey = y - v[1] * d, ez = z - v[2] * d;
+    const float cx = A[0] * ex + A[1] * ey + A[2] * ez, cy = A[1] * ex + A[3] * ey + A[4] * ez,
+                cz = A[2] * ex + A[4] * ey + A[5] * ez;
     c.L += wide_double(d);
-    c.u[0] += wide_double(A[0] * ex + A[1] * ey + A[2] * ez);
-    c.u[1] += wide_double(A[1] * ex + A[3] * ey + A[4] * ez);
-    c.u[2] += wide_double(A[2] * ex + A[4] * ey + A[5] * ez);
-    if (it >= 1 && !(fabsf(d) > 1e-12f * l)) break;
+    c.u[0] += wide_double(cx);
+    c.u[1] += wide_double(cy);
+    c.u[2] += wide_double(cz);
+    settled = fabsf(d) <= 1e-12f * l && fabsf(cx) + fabsf(cy) + fabsf(cz) <= 1e-11f * w;
+    if (it >= 1 && settled) break;
+  }
+  bool good = true;
+  if (__builtin_expect(!(settled && det > 0.f && w > 0.f), 0)) {
+    double q[10] = {T00, t[0], t[1], t[2], S[0], S[1], S[2], S[3], S[4], S[5]};
+    good = settle_frame(q);
+    c.L = q[0];
+    c.u[0] = q[1];
+    c.u[1] = q[2];
+    c.u[2] = q[3];
   }
   const double w2 = fma(-c.u[2], c.u[2], fma(-c.u[1], c.u[1], fma(-c.u[0], c.u[0], 1.0)));
   c.U0 = reciprocal_sqrt(w2);
   c.n = c.U0 * fma(-c.u[2], N[3], fma(-c.u[1], N[2], fma(-c.u[0], N[1], N[0])));
-  c.fL = cut_float(c.L);
-  c.fn = cut_float(c.n);
-  c.ok = det > 0.f && w > 0.f && __double2hiint(w2) > 0 && c.fn > 0.f && c.fL > 0.f && c.fL < 1e30f && c.fn < 1e30f &&
-         c.fn > 1e-30f && c.fL > 1e-30f;
+  c.ok = good && __double2hiint(w2) > 0 && between(c.n, -100, 100) && between(c.L, -100, 100);
   return c;
 }
 
@@ -463,7 +474,7 @@ __global__ void __launch_bounds__(128, ORDER == 2 ? 6 : 5) k_step3x(const __grid
 // Fields of f(t): the populations pulled from f*(t-1) (after a step) or, at
 // t = 0, f*(0) = f^eq itself: n, ux, uy, uz, T, eps (n NaN without a Landau frame).
 template <int ORDER, typename S>
-__global__ void __launch_bounds__(128) k_fields3x(const __grid_constant__ Tables3x<ORDER> tb,
+__global__ void __launch_bounds__(128, ORDER == 2 ? 7 : 6) k_fields3x(const __grid_constant__ Tables3x<ORDER> tb,
                                                   const __grid_constant__ Fields3Args<S> a) {
   const Scalars3& s = a.s;
   const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 4 + threadIdx.y, z = blockIdx.z;

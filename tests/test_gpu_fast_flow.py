@@ -1,0 +1,96 @@
+"""Fast flows.  The Landau frame of a flow of Lorentz factor g is what remains of a
+tensor g^2 times as large, so that a relative rounding e of T^ab changes eps by
+about g^4 e and u by g^2 e; with populations of both signs e is 2^-53 (the stored
+values being given) times k = sum |f| p0^2 / T^00.  The bars are 16 times
+that, for the oracle's rounding and the library's together."""
+import numpy as np
+import pytest
+
+from oracle import d3 as OD
+from tests.cases import rel_linf
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rl():
+    from paper_1909_04502_gb300 import rlbm
+    return rlbm
+
+
+def _order3(lat, quad):
+    pos = {(tuple(v), round(p, 9)): i for i, (v, p) in enumerate(zip(lat.n.tolist(), lat.p[:, 0]))}
+    return [pos[(tuple(v), round(p, 9))] for v, p in zip(quad.n.tolist(), quad.p[:, 0])]
+
+
+def _bar(f, quad, u):
+    p2 = (quad.p[:, 0] ** 2).reshape(-1, 1, 1, 1)
+    k = float(((np.abs(f) * p2).sum(0) / (f * p2).sum(0)).max())
+    return 16 * k * 2.0 ** -53 / (1 - u * u) ** 2
+
+
+def _check_fields3(mo, want, bar, u):
+    assert np.isfinite(mo["n"]).all()
+    for name, w in (("n", want.n), ("T", want.T), ("eps", want.eps)):
+        assert np.abs(mo[name] / w - 1).max() <= bar
+    for k, name in ((1, "ux"), (2, "uy"), (3, "uz")):
+        assert np.abs(mo[name] - want.u(k)).max() <= bar * (1 - u * u)
+
+
+@pytest.mark.parametrize("order,precision,speeds", [
+    (2, "fp64", (0.9, 0.95, 0.99, 0.993, 0.995, 0.999, 0.9995)), (3, "fp64", (0.9, 0.95, 0.99, 0.995, 0.999, 0.9995)),
+    (2, "fp32", (0.9, 0.99, 0.995, 0.999)), (3, "fp32", (0.9, 0.99, 0.993))])
+def test_fields3_of_fast_cells(rl, order, precision, speeds):
+    """Cells of one speed and random directions: the fields of the stored populations."""
+    quad = OD.massless_quadrature_3d(order)
+    shape = (6, 7, 33)
+    for u in speeds:
+        rng = np.random.default_rng(order)
+        v = rng.standard_normal((3,) + shape)
+        v *= u / np.sqrt((v * v).sum(0))
+        lat = rl.Lattice3(33, 7, 6, tau=0.8, precision=precision, order=order)
+        lat.init(1 + 0.3 * rng.random(shape), *[np.ascontiguousarray(a) for a in v], 1 + 0.2 * rng.random(shape))
+        f = lat.populations()[_order3(lat, quad)]
+        _check_fields3(lat.moments(), OD.macroscopic3(f, quad), _bar(f, quad, u), u)
+        lat.close()
+
+
+def _mj_moments3(order, U):
+    """Maxwell-Juttner moments of the basis 1 | p0 p | p0 pi, pi pj | p0 pi pj,
+    pi pj pk at n = T = 1 (App. B, d = 3, m = 0), in the order of plan3's H."""
+    eta = np.diag([1.0, -1, -1, -1])
+    two = [(0, i) for i in (1, 2, 3)] + [(i, j) for i in (1, 2, 3) for j in range(i, 4)]
+    M = [0.5] + list(U) + [4 * U[a] * U[b] - eta[a, b] for a, b in two]
+    if order == 3:
+        pairs = [(i, j) for i in (1, 2, 3) for j in range(i, 4)]
+        for a, b, c in [(0,) + p for p in pairs] + [(i, j, k) for i, j in pairs for k in range(j, 4)]:
+            M.append(24 * U[a] * U[b] * U[c] - 4 * (eta[a, b] * U[c] + eta[a, c] * U[b] + eta[b, c] * U[a]))
+    return np.array(M)
+
+
+@pytest.mark.parametrize("order", [2, 3])
+@pytest.mark.parametrize("u", [0.9, 0.95, 0.99, 0.995, 0.999])
+def test_step3_of_a_uniform_stream(rl, order, u):
+    """A uniform equilibrium stream: a step of its stored populations against the
+    oracle's.  The bar is the oracle's amplification of rounding errors of the
+    terms H_ik M_k (e sum_k |H_ik M_k| of either sign, e = 2^-40, the largest of 64
+    draws), at 16 roundings: 16 times that at e = 2^-53."""
+    plan = rl.plan3(order)
+    nx, ny, nz = 34, 7, 6
+    one = np.ones((nz, ny, nx))
+    v = u * np.array([2.0, -1.0, 0.5]) / np.sqrt(5.25)
+    lat = rl.Lattice3(nx, ny, nz, tau=0.8, precision="fp64", order=order)
+    lat.init(one, *[c * one for c in v], one)
+    f = lat.populations()
+    quad = OD.massless_quadrature_3d(order)
+    idx = _order3(lat, quad)
+    HM = np.abs(plan["H"] * _mj_moments3(order, np.concatenate([[1.0], v]) / np.sqrt(1 - u * u))).sum(1)[idx, None]
+    draws = f[idx, 0, 0, :1] + 2.0 ** -40 * HM * np.sign(np.random.default_rng(1).random((lat.Q, 65)) - 0.5)
+    draws[:, 0] = f[idx, 0, 0, 0]
+    fs, fields = OD.collide3(draws, quad, OD.Expansion3(quad, order), 0.8)
+    assert fields.ok.all()
+    bar = 16 * 2.0 ** (40 - 53) * rel_linf(fs[:, 1:], fs[:, :1])
+    lat.step(1)
+    assert lat.sync_status() == (0, 0)
+    assert rel_linf(lat.populations()[idx], fs[:, :1, None, None]) <= bar
+    lat.close()
