@@ -84,9 +84,9 @@ __device__ __forceinline__ Cell2 landau2x(const double (&v)[9], float k, double 
     const double r = fma(e, e, 4.0 * m * (e - m)), y = reciprocal_sqrt(r), q = r * y;
     c.T = 0.25 * ((e - 2.0 * m) + fma(0.5 * y, fma(-q, q, r), q));
   }
-  const float fn = cut_float(c.n), fL = cut_float(c.L), fTm = cut_float(c.T);
-  c.ok = det > 0.f && w > 0.f && __double2hiint(w2) > 0 && fn > 1e-30f && fn < 1e30f && fL > 1e-30f && fL < 1e30f &&
-         fTm > 0.f && fTm < 3e38f;
+  // (NaN where the massive EOS has no real temperature: eps / n below 0.83 m)
+  c.ok = det > 0.f && w > 0.f && __double2hiint(w2) > 0 && between(c.n, -100, 100) && between(c.L, -100, 100) &&
+         between(c.T, -1022, 127);
   return c;
 }
 
