@@ -35,7 +35,8 @@ struct Cell2 {
 };
 
 // As landau3x: the root and u in FP32 by Newton on the secular equation, then
-// (l, u) by iterative refinement with FP64 residuals; T from the d = 2 EOS.
+// (l, u) by iterative refinement with FP64 residuals, and in FP64 (frame64.cuh)
+// what has not settled after six passes; T from the d = 2 EOS.
 template <bool MASSLESS>
 __device__ __forceinline__ Cell2 landau2x(const double (&v)[9], float k, double m) {
   const float fT = cut_float(v[3]), f0 = cut_float(v[4]), f1 = cut_float(v[5]);
@@ -61,6 +62,7 @@ __device__ __forceinline__ Cell2 landau2x(const double (&v)[9], float k, double 
   c.u[0] = wide_double(u0);
   c.u[1] = wide_double(u1);
   const float iw = __fdividef(1.f, w), Axx = yy * id, Ayy = xx * id, Axy = -fxy * id;
+  bool settled = false;
 #pragma unroll 1
   for (int it = 0; it < 6; ++it) {
     const double r0 = fma(-v[5], c.u[1], fma(-v[4], c.u[0], v[3] - c.L));
@@ -69,10 +71,20 @@ __device__ __forceinline__ Cell2 landau2x(const double (&v)[9], float k, double 
     const float x = cut_float(rx), y = cut_float(ry);
     const float d = (cut_float(r0) - u0 * x - u1 * y) * iw;
     const float ex = x - u0 * d, ey = y - u1 * d;
+    const float cx = Axx * ex + Axy * ey, cy = Axy * ex + Ayy * ey;
     c.L += wide_double(d);
-    c.u[0] += wide_double(Axx * ex + Axy * ey);
-    c.u[1] += wide_double(Axy * ex + Ayy * ey);
-    if (it >= 1 && !(fabsf(d) > 1e-12f * l)) break;
+    c.u[0] += wide_double(cx);
+    c.u[1] += wide_double(cy);
+    settled = fabsf(d) <= 1e-12f * l && fabsf(cx) + fabsf(cy) <= 1e-11f * w;
+    if (it >= 1 && settled) break;
+  }
+  bool good = true;
+  if (__builtin_expect(!(settled && det > 0.f && w > 0.f), 0)) {
+    double q[10] = {v[3], v[4], v[5], 0.0, v[6], v[7], 0.0, v[8], 0.0, 0.0};
+    good = settle_frame(q);
+    c.L = q[0];
+    c.u[0] = q[1];
+    c.u[1] = q[2];
   }
   const double w2 = fma(-c.u[1], c.u[1], fma(-c.u[0], c.u[0], 1.0));
   c.U0 = reciprocal_sqrt(w2);
@@ -85,7 +97,7 @@ __device__ __forceinline__ Cell2 landau2x(const double (&v)[9], float k, double 
     c.T = 0.25 * ((e - 2.0 * m) + fma(0.5 * y, fma(-q, q, r), q));
   }
   // (NaN where the massive EOS has no real temperature: eps / n below 0.83 m)
-  c.ok = det > 0.f && w > 0.f && __double2hiint(w2) > 0 && between(c.n, -100, 100) && between(c.L, -100, 100) &&
+  c.ok = good && __double2hiint(w2) > 0 && between(c.n, -100, 100) && between(c.L, -100, 100) &&
          between(c.T, -1022, 127);
   return c;
 }
@@ -273,7 +285,7 @@ constexpr size_t shared2x(int K, int mode, int Q) {
 }
 
 template <int K, int MODE, bool MASSLESS>
-__global__ void __launch_bounds__(kThreads2x, K == 9 ? 5 : 4) k_step2x(const __grid_constant__ Tables2x tb,
+__global__ void __launch_bounds__(kThreads2x, K == 9 || MODE == kOnLattice ? 5 : 4) k_step2x(const __grid_constant__ Tables2x tb,
                                                                         const __grid_constant__ StepArgs<double> a,
                                                                         double inv_tau) {
   extern __shared__ int2 columns[];
@@ -476,7 +488,7 @@ dim3 grid2x(const Scalars& s, dim3 block) { return dim3((s.nx + block.x - 1) / b
 
 // Fields of f(t) (the populations streamed from f*(t-1), or f*(0) in place).
 template <int MODE, bool MASSLESS>
-__global__ void __launch_bounds__(kThreads2x) k_fields2x(const __grid_constant__ Tables2x tb,
+__global__ void __launch_bounds__(kThreads2x, 8) k_fields2x(const __grid_constant__ Tables2x tb,
                                                          const __grid_constant__ MomentArgs<double> a) {
   const Scalars& s = a.s;
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;

@@ -7,7 +7,9 @@ import numpy as np
 import pytest
 
 from oracle import d3 as OD
-from tests.cases import rel_linf
+from oracle import lattice as OL
+from oracle import scheme as OS
+from tests.cases import oracle_quadrature, permutation, rel_linf
 
 pytestmark = pytest.mark.gpu
 
@@ -24,7 +26,7 @@ def _order3(lat, quad):
 
 
 def _bar(f, quad, u):
-    p2 = (quad.p[:, 0] ** 2).reshape(-1, 1, 1, 1)
+    p2 = (quad.p[:, 0] ** 2).reshape((-1,) + (1,) * (f.ndim - 1))
     k = float(((np.abs(f) * p2).sum(0) / (f * p2).sum(0)).max())
     return 16 * k * 2.0 ** -53 / (1 - u * u) ** 2
 
@@ -55,17 +57,13 @@ def test_fields3_of_fast_cells(rl, order, precision, speeds):
         lat.close()
 
 
-def _mj_moments3(order, U):
-    """Maxwell-Juttner moments of the basis 1 | p0 p | p0 pi, pi pj | p0 pi pj,
-    pi pj pk at n = T = 1 (App. B, d = 3, m = 0), in the order of plan3's H."""
-    eta = np.diag([1.0, -1, -1, -1])
-    two = [(0, i) for i in (1, 2, 3)] + [(i, j) for i in (1, 2, 3) for j in range(i, 4)]
-    M = [0.5] + list(U) + [4 * U[a] * U[b] - eta[a, b] for a, b in two]
-    if order == 3:
-        pairs = [(i, j) for i in (1, 2, 3) for j in range(i, 4)]
-        for a, b, c in [(0,) + p for p in pairs] + [(i, j, k) for i, j in pairs for k in range(j, 4)]:
-            M.append(24 * U[a] * U[b] * U[c] - 4 * (eta[a, b] * U[c] + eta[a, c] * U[b] + eta[b, c] * U[a]))
-    return np.array(M)
+def _draws(H, f):
+    """f = H M, and 64 times with errors 2^-40 sum_k |H_ik M_k| of random sign."""
+    M = np.linalg.lstsq(H, f, rcond=None)[0]
+    out = f[:, None] + 2.0 ** -40 * np.abs(H * M).sum(1)[:, None] * np.sign(
+        np.random.default_rng(1).random((len(f), 65)) - 0.5)
+    out[:, 0] = f
+    return out
 
 
 @pytest.mark.parametrize("order", [2, 3])
@@ -84,13 +82,52 @@ def test_step3_of_a_uniform_stream(rl, order, u):
     f = lat.populations()
     quad = OD.massless_quadrature_3d(order)
     idx = _order3(lat, quad)
-    HM = np.abs(plan["H"] * _mj_moments3(order, np.concatenate([[1.0], v]) / np.sqrt(1 - u * u))).sum(1)[idx, None]
-    draws = f[idx, 0, 0, :1] + 2.0 ** -40 * HM * np.sign(np.random.default_rng(1).random((lat.Q, 65)) - 0.5)
-    draws[:, 0] = f[idx, 0, 0, 0]
+    draws = _draws(plan["H"], f[:, 0, 0, 0])[idx]
     fs, fields = OD.collide3(draws, quad, OD.Expansion3(quad, order), 0.8)
     assert fields.ok.all()
     bar = 16 * 2.0 ** (40 - 53) * rel_linf(fs[:, 1:], fs[:, :1])
     lat.step(1)
     assert lat.sync_status() == (0, 0)
     assert rel_linf(lat.populations()[idx], fs[:, :1, None, None]) <= bar
+    lat.close()
+
+
+GASES = [(0.0, 2), (0.0, 3), (1.0, 2), (5.0, 3)]
+
+
+@pytest.mark.parametrize("m,order", GASES)
+def test_fields2_of_fast_cells(rl, m, order):
+    """As in (3+1)-d; T follows eps / n with a factor of at most eps / (n T)."""
+    for u in (0.9, 0.95, 0.99, 0.995, 0.998, 0.999):
+        rng = np.random.default_rng(order)
+        th, shape = rng.uniform(0, 2 * np.pi, (7, 33)), (7, 33)
+        lat = rl.Lattice(33, 7, m=m, order=order, tau=0.8, precision="fp64")
+        quad = oracle_quadrature(m, order, lat.n, rl.plan(m=m, order=order)["v0"])
+        lat.init(1 + 0.3 * rng.random(shape), u * np.cos(th), u * np.sin(th), 1 + 0.2 * rng.random(shape))
+        f = lat.populations()[permutation(lat.n, lat.p, quad)]
+        want, mo, bar = OS.macroscopic(f, quad), lat.moments(), _bar(f, quad, u)
+        assert lat.sync_status() == (0, 0)
+        assert np.abs(mo["n"] / want.n - 1).max() <= bar and np.abs(mo["eps"] / want.eps - 1).max() <= bar
+        assert np.abs(mo["T"] / want.T - 1).max() <= bar * (want.eps / (want.n * want.T)).max()
+        for k, name in ((1, "ux"), (2, "uy")):
+            assert np.abs(mo[name] - want.U[k] / want.U[0]).max() <= bar * (1 - u * u)
+        lat.close()
+
+
+@pytest.mark.parametrize("m,order", GASES)
+@pytest.mark.parametrize("u", [0.9, 0.99, 0.995, 0.999])
+def test_step2_of_a_uniform_stream(rl, m, order, u):
+    plan = rl.plan(m=m, order=order)
+    one = np.ones((6, 34))
+    lat = rl.Lattice(34, 6, m=m, order=order, tau=0.8, precision="fp64")
+    quad = oracle_quadrature(m, order, lat.n, plan["v0"])
+    idx = permutation(lat.n, lat.p, quad)
+    lat.init(one, 0.8 * u * one, -0.6 * u * one, one)
+    draws = _draws(plan["H"], lat.populations()[:, 0, 0])[idx][:, :, None]
+    fs, fields = OS.collide(draws, quad, OL.Expansion(quad), 0.8)
+    assert fields.ok.all()
+    bar = 16 * 2.0 ** (40 - 53) * rel_linf(fs[:, 1:], fs[:, :1])
+    lat.step(1)
+    assert lat.sync_status() == (0, 0)
+    assert rel_linf(lat.populations()[idx], fs[:, :1]) <= bar
     lat.close()
