@@ -284,6 +284,45 @@ constexpr size_t shared2x(int K, int mode, int Q) {
   return (size_t)(K + 4 + (kept2x(K, mode) ? Q : 0)) * kThreads2x * 8;
 }
 
+// The relaxation in FP64, for a cell whose rate or equilibrium the fixed point does
+// not hold (a tau of its field that is zero, NaN or below 1/64, say), or
+// that has no frame and keeps its populations.  v: K basis moments times 2^hk in units
+// of 2^E, then tau^-1 U0 and vscale tau^-1 U^i (a column of the shared memory); kept:
+// the streamed populations, or null where they are read again.
+template <int K>
+__device__ __noinline__ void relax_plain2(const Tables2x& tb, const StepArgs<double>& a, const double* v, const double* kept,
+                                          const double* base, int E, int x, int y) {
+  const Scalars& s = a.s;
+  const double o0 = v[K * kThreads2x], kx = v[(K + 1) * kThreads2x], ky = v[(K + 2) * kThreads2x];
+  // sx, sy: the signs of the odd members of p^x and p^y, 0 where the row has none
+  auto relax = [&](int i, const Cx* H, double sx, double sy, double om, int e) {
+    double sum = 0.0;
+#pragma unroll 1
+    for (int k = 0; k < K; ++k) {
+      const double c = (double)(((long long)H[k].h << 32) + H[k].l);
+      sum = fma((mono_ax(k) ? sx : 1.0) * (mono_ay(k) ? sy : 1.0) * c, v[k * kThreads2x], sum);
+    }
+    const double f = kept ? kept[i * kThreads2x] : __ldg(base + tb.off[i]);
+    const double g = fma(om, scaled(sum, E - 1023 + e - kCoefH) - f, f);
+    a.fout[(base - a.fin) + (long long)i * s.iplane] = g;
+    for_each_halo_image(s, x, y, [&](long long hi) { a.fout[hi + (long long)i * s.iplane] = g; });
+  };
+#pragma unroll 1
+  for (int q = 0; q < 4 * tb.nq; ++q) {
+    const int r = q >> 2;
+    const double sx = (q & 1) ? -1.0 : 1.0, sy = (q & 2) ? -1.0 : 1.0;
+    relax(tb.firstq[r] + (q & 3), tb.Hq[r], sx, sy, o0 - sx * tb.nq_x[r] * kx - sy * tb.nq_y[r] * ky, tb.erq[r] + tb.rhoq[r]);
+  }
+#pragma unroll 1
+  for (int q = 0; q < 4 * tb.na; ++q) {
+    const int r = q >> 2, along = (q >> 1) & 1;
+    const double sg = (q & 1) ? -1.0 : 1.0;
+    relax(tb.firsta[r] + (q & 3), tb.Ha[r][along], along ? 0.0 : sg, along ? sg : 0.0,
+          o0 - sg * tb.na_x[r] * (along ? ky : kx), tb.era[r] + tb.rhoa[r]);
+  }
+  if (tb.nr) relax(tb.firstr, tb.Hr, 0.0, 0.0, o0, tb.err + tb.rhor);
+}
+
 template <int K, int MODE, bool MASSLESS>
 __global__ void __launch_bounds__(kThreads2x, K == 9 || MODE == kOnLattice ? 5 : 4) k_step2x(const __grid_constant__ Tables2x tb,
                                                                         const __grid_constant__ StepArgs<double> a,
@@ -314,7 +353,6 @@ __global__ void __launch_bounds__(kThreads2x, K == 9 || MODE == kOnLattice ? 5 :
 
   int uf, ue, eo;            // the unit 2^(u - kBits) of a quartet: u = max(its exponent + uf, rho + ue)
   long long O0, W[2];        // tau^-1 U0 and vscale tau^-1 U^i in units of 2^(eo - 62)
-  bool ok;
   {
     long long m[9];
     int E;
@@ -323,7 +361,7 @@ __global__ void __launch_bounds__(kThreads2x, K == 9 || MODE == kOnLattice ? 5 :
 #pragma unroll
     for (int j = 0; j < 9; ++j) v[j] = from_fixed(m[j], 1023 + tb.sk[j] - kBitsM4 + 64 - kCoefM);
     const Cell2 c = landau2x<MASSLESS>(v, s.kappa_guess, s.m);
-    ok = c.ok && E > 128 && E < 2040;
+    const bool ok = c.ok && E > 128 && E < 2040;
     const double Ux = c.u[0] * c.U0, Uy = c.u[1] * c.U0;
     double Mk[K], lo[K];
     mj_moments2x<K, MASSLESS>(c, Ux, Uy, s.m, Mk, lo);
@@ -338,9 +376,26 @@ __global__ void __launch_bounds__(kThreads2x, K == 9 || MODE == kOnLattice ? 5 :
     if (s.tau_mode == 1) it = 1.0 / chained(a.tau_field)[y * s.nx + x];
     else if (s.tau_mode == 2) it = c.T / s.tau_coef;
     else it = inv_tau;
-    const double o0 = it * c.U0;
+    const double o0 = it * c.U0, kl = it * tb.vscale;
     const int xg = above(sum), xo = above(2.f * fabsf(cut_float(o0)));
-    ok = ok && xg < 60 && xg > -60;
+    // (a population's unit leaves room for rate times population: with rates from 64 on
+    // less than FP64 would be left of it)
+    const bool rate = (__double2hiint(o0) & 0x7FFFFFFF) < (1023 + 6) << 20;      // finite, |o0| < 2^6
+    if (__builtin_expect(!(ok && rate && xg < 60 && xg > -60), 0)) {
+      // no Landau frame: counted, left unrelaxed (a population that is not finite becomes NaN)
+      if (!ok) atomicAdd(a.status, 1ULL);
+      double* const v = (double*)M.s;
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const double f = has_lo<K, MASSLESS>(k) ? Mk[k] + lo[k] : Mk[k];
+        v[k * kThreads2x] = ok ? f * __hiloint2double((1023 + tb.hk[k]) << 20, 0) : 0.0;
+      }
+      v[K * kThreads2x] = ok ? o0 : 0.0;
+      v[(K + 1) * kThreads2x] = ok ? kl * Ux : 0.0;
+      v[(K + 2) * kThreads2x] = ok ? kl * Uy : 0.0;
+      relax_plain2<K>(tb, a, v, kept2x(K, MODE) ? F : nullptr, base, ok ? E : 1023, x, y);
+      return;
+    }
     uf = max(0, xo - 2);
     ue = E + xg + max(0, xo - 3);
 #pragma unroll
@@ -351,20 +406,8 @@ __global__ void __launch_bounds__(kThreads2x, K == 9 || MODE == kOnLattice ? 5 :
     }
     eo = max(xo, -2);
     O0 = scaled_integer(o0, 62 - eo);
-    const double kl = it * tb.vscale;
     W[0] = scaled_integer(kl * Ux, 62 - eo);
     W[1] = scaled_integer(kl * Uy, 62 - eo);
-  }
-  if (!ok) {
-    // no Landau frame: counted, left unrelaxed (a population that is not finite becomes NaN)
-    atomicAdd(a.status, 1ULL);
-#pragma unroll 1
-    for (int i = 0; i < tb.Q; ++i) {
-      const double f = again(i), g = fma(0.0, -f, f);
-      ob[i * P] = g;
-      for_each_halo_image(s, x, y, [&](long long hi) { a.fout[hi + (long long)i * P] = g; });
-    }
-    return;
   }
   const bool edge = (s.boundary == 0 ? (x < s.hx || x >= s.nx - s.hx) : (x == 0 || x == s.nx - 1)) || y < s.hy ||
                     y >= s.ny - s.hy;

@@ -5,7 +5,9 @@ computed in FP64 or counted."""
 import numpy as np
 import pytest
 
-from tests.cases import rel_linf
+from oracle import lattice as OL
+from oracle import scheme as OS
+from tests.cases import oracle_quadrature, permutation, rel_linf
 
 pytestmark = pytest.mark.gpu
 
@@ -61,4 +63,38 @@ def test_frames_without_a_temperature_are_counted(rl, order):
         lat.step(1)
         assert lat.sync_status(raise_on_error=False) == (-4, nx * ny)
         assert np.array_equal(lat.populations(), G)
+    lat.close()
+
+
+@pytest.mark.parametrize("m,order,stream", [(0.0, 2, "onlattice"), (5.0, 3, "onlattice"), (0.0, 3, "bilinear"),
+                                            (1.0, 2, "bilinear")])
+def test_relaxation_time_fields_of_any_value(rl, m, order, stream):
+    """tau of 0, NaN, infinity, a negative one and some far below and above one, in an
+    interior cell, at an edge and in a corner each: what the oracle's FP64 relaxation
+    gives, to 1e-12 of f (1 + 1/tau); not finite where it is not."""
+    nx, ny = 35, 9
+    lam = 0.9 if stream == "bilinear" else 0.0
+    lat = rl.Lattice(nx, ny, m=m, order=order, tau_mode="field", precision="fp64", stream=stream, lam=lam)
+    quad = oracle_quadrature(m, order, lat.n, rl.plan(m=m, order=order)["v0"])
+    idx = permutation(lat.n, lat.p, quad)
+    rng = np.random.default_rng(order)
+    lat.init(1 + 0.3 * rng.random((ny, nx)), *(0.2 * rng.random((2, ny, nx)) - 0.1), 1 + 0.1 * rng.random((ny, nx)))
+    f = lat.populations()[idx]
+    f = OS.stream_onlattice(f, quad.n) if stream == "onlattice" else OS.stream_bilinear(f, lam * quad.velocity(), "periodic")
+    odd = [0.0, np.nan, np.inf, -1.0, 1e-12, 2.0 ** -26.5, 2.0 ** -28.5, 1e-5, 1e5, 1e300, 5e-324]
+    for at in ([4] * len(odd), [0] * len(odd), [ny - 1] * len(odd)):
+        tau = np.full((ny, nx), 0.9)
+        tau[at, (np.arange(len(odd)) * 3) % nx] = odd
+        with np.errstate(all="ignore"):
+            want = OS.collide(f, quad, OL.Expansion(quad), tau)[0]
+            bar = 1e-12 * np.abs(f).max() * (1 + 1 / np.abs(tau))
+        start = lat.populations()
+        lat.set_tau_field(tau)
+        lat.step(1)
+        got = lat.populations()[idx]
+        assert lat.sync_status() == (0, 0)
+        ok = np.isfinite(want).all(0)
+        assert (~ok).sum() == 3 and np.array_equal(np.isfinite(got).all(0), ok)
+        assert (np.abs(got - want).max(0)[ok] <= bar[ok]).all()
+        lat.set_populations(start)
     lat.close()
