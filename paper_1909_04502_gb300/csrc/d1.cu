@@ -244,6 +244,20 @@ __device__ __forceinline__ Cell1 macro1x(const Tab1x<N>& tb, const S (&g)[2 * N]
   return c;
 }
 
+// The relaxation of one direction in FP64, for the cells whose rate or equilibrium
+// the fixed point does not hold.  v: the N populations (replaced), then the moments n T2^(a-1)
+// e^(+-a theta) in units of 2^E.  Out of line, in memory.
+template <int N>
+__device__ __noinline__ void relax_plain1(const Tab1x<N>& tb, double* v, int E, double om) {
+  for (int j = 0; j < N; ++j) {
+    double sum = 0.0;
+    for (int a = 0; a < N; ++a)
+      sum = fma(rlbm::constant_value(tb.H[j][a], tb.hk[a]), v[N + a], sum);
+    const double feq = rlbm::scaled(sum, E - 1023 + tb.er[j] + tb.rho[j] - rlbm::kCoefH);
+    v[j] = om == 1.0 ? feq : fma(om, feq - v[j], v[j]);
+  }
+}
+
 template <int N>
 __global__ void __launch_bounds__(kThreads) k_step1x(const __grid_constant__ Tab1x<N> tb, const __grid_constant__ Sc s,
                                                      const double* __restrict__ before, double* __restrict__ fout,
@@ -272,7 +286,9 @@ __global__ void __launch_bounds__(kThreads) k_step1x(const __grid_constant__ Tab
     c.eth[0] = c.eth[1] = om[0] = om[1] = 1.0;
   }
   const int xo = above(fmaxf(cut_float(om[0]), cut_float(om[1]))), eo = max(xo, -2), uf = max(0, xo - 2);
-  const long long half = 1LL << (29 - eo);
+  const long long half = 1LL << max(29 - eo, 0);
+  // (moments within the float range, and, as in step2x.cu, rates below 64)
+  const bool fits = between(c.n, -28, 28) && between(c.T2, -28, 12) && between(c.eth[0], -8, 8) && xo <= 6;
 #pragma unroll
   for (int d = 0; d < 2; ++d) {
     double m[N];
@@ -285,6 +301,15 @@ __global__ void __launch_bounds__(kThreads) k_step1x(const __grid_constant__ Tab
       sum += cut_float(m[a]) * __uint_as_float((unsigned)(127 + tb.hk[a]) << 23);
     }
     const int xg = above(sum), sE = c.E + xg, ue = sE + max(0, xo - 3);
+    if (__builtin_expect(!(fits && xg < 60 && xg > -60), 0)) {
+      double v[2 * N];
+#pragma unroll
+      for (int a = 0; a < N; ++a) v[a] = g[2 * a + d], v[N + a] = m[a];
+      relax_plain1<N>(tb, v, c.E, om[d]);
+#pragma unroll
+      for (int a = 0; a < N; ++a) g[2 * a + d] = v[a];
+      continue;
+    }
     int vh[N], vl[N];
 #pragma unroll
     for (int a = 0; a < N; ++a) {

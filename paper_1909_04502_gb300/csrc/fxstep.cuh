@@ -77,6 +77,11 @@ __device__ __forceinline__ bool between(double v, int lo, int hi) {
   return (unsigned)(__double2hiint(v) - ((1023 + lo) << 20)) < (unsigned)((hi - lo) << 20);
 }
 
+// a table constant, as the integer that it stands for, times 2^k
+__device__ __forceinline__ double constant_value(Cx c, int k) {
+  return (double)(((long long)c.h << 32) + c.l) * __hiloint2double((1023 + k) << 20, 0);
+}
+
 // frame64 out of line: v = T00, T0i, Txx Txy Txz Tyy Tyz Tzz becomes l, u; in
 // memory, so that the caller holds no registers for them.
 __device__ __noinline__ bool settle_frame(double* v) {

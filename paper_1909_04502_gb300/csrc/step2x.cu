@@ -285,10 +285,10 @@ constexpr size_t shared2x(int K, int mode, int Q) {
 }
 
 // The relaxation in FP64, for a cell whose rate or equilibrium the fixed point does
-// not hold (a tau of its field that is zero, NaN or below 1/64, say), or
-// that has no frame and keeps its populations.  v: K basis moments times 2^hk in units
-// of 2^E, then tau^-1 U0 and vscale tau^-1 U^i (a column of the shared memory); kept:
-// the streamed populations, or null where they are read again.
+// not hold (a tau of its field that is zero, NaN or below 1/64, say), or that has no
+// frame and keeps its populations.  v: K basis moments in units of 2^E, then
+// tau^-1 U0 and vscale tau^-1 U^i (a column of the shared memory); kept: the
+// streamed populations, or null where they are read again.
 template <int K>
 __device__ __noinline__ void relax_plain2(const Tables2x& tb, const StepArgs<double>& a, const double* v, const double* kept,
                                           const double* base, int E, int x, int y) {
@@ -299,8 +299,7 @@ __device__ __noinline__ void relax_plain2(const Tables2x& tb, const StepArgs<dou
     double sum = 0.0;
 #pragma unroll 1
     for (int k = 0; k < K; ++k) {
-      const double c = (double)(((long long)H[k].h << 32) + H[k].l);
-      sum = fma((mono_ax(k) ? sx : 1.0) * (mono_ay(k) ? sy : 1.0) * c, v[k * kThreads2x], sum);
+      sum = fma((mono_ax(k) ? sx : 1.0) * (mono_ay(k) ? sy : 1.0) * constant_value(H[k], tb.hk[k]), v[k * kThreads2x], sum);
     }
     const double f = kept ? kept[i * kThreads2x] : __ldg(base + tb.off[i]);
     const double g = fma(om, scaled(sum, E - 1023 + e - kCoefH) - f, f);
@@ -381,14 +380,16 @@ __global__ void __launch_bounds__(kThreads2x, K == 9 || MODE == kOnLattice ? 5 :
     // (a population's unit leaves room for rate times population: with rates from 64 on
     // less than FP64 would be left of it)
     const bool rate = (__double2hiint(o0) & 0x7FFFFFFF) < (1023 + 6) << 20;      // finite, |o0| < 2^6
-    if (__builtin_expect(!(ok && rate && xg < 60 && xg > -60), 0)) {
+    // (moments within the float range, whatever U and T within these)
+    const bool fits = between(c.n, -28, 28) && between(c.L, -28, 28) && between(c.T, -30, 24) && between(c.U0, -1, 10);
+    if (__builtin_expect(!(ok && rate && fits && xg < 60 && xg > -60), 0)) {
       // no Landau frame: counted, left unrelaxed (a population that is not finite becomes NaN)
       if (!ok) atomicAdd(a.status, 1ULL);
       double* const v = (double*)M.s;
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         const double f = has_lo<K, MASSLESS>(k) ? Mk[k] + lo[k] : Mk[k];
-        v[k * kThreads2x] = ok ? f * __hiloint2double((1023 + tb.hk[k]) << 20, 0) : 0.0;
+        v[k * kThreads2x] = ok ? f : 0.0;
       }
       v[K * kThreads2x] = ok ? o0 : 0.0;
       v[(K + 1) * kThreads2x] = ok ? kl * Ux : 0.0;

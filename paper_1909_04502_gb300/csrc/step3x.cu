@@ -299,6 +299,48 @@ __device__ __forceinline__ void mj_moments3x(const Cell3& c, const double (&U)[3
   }
 }
 
+// The relaxation in FP64, for a cell whose rate or equilibrium the fixed point does
+// not hold (gamma of about 64 and above), or that has no frame and keeps its populations.
+// v: K basis moments in units of 2^E, then tau^-1 U0 and tau^-1 U^i / |n| (a
+// column of the shared memory).
+template <int ORDER>
+__device__ __noinline__ void relax_plain3(const Tables3x<ORDER>& tb, const Step3Args<double>& a, const double* v, int E,
+                                          int x, int y, int z) {
+  using T = Tables3x<ORDER>;
+  const Scalars3& s = a.s;
+  const long long si = sidx3(s, x, y, z);
+  long long img[26];
+  const int nimg = cell_images(s, x, y, z, img);
+  // the member of a run that negates the components of neg
+  auto relax = [&](int i, int off, const Cx* H, const int* n, int mask, int neg, int e) {
+    double sum = 0.0, om = v[T::K * 128];
+#pragma unroll 1
+    for (int k = 0; k < T::K; ++k)
+      if (!(kPar3[k] & ~mask))
+        sum = fma((__popc(kPar3[k] & neg) & 1) ? -v[k * 128] : v[k * 128], constant_value(H[k], tb.hk[k]), sum);
+    for (int c = 0; c < 3; ++c)
+      if (mask >> c & 1) om = fma((neg >> c & 1) ? (double)n[c] : -(double)n[c], v[(T::K + 1 + c) * 128], om);
+    const long long p = (long long)i * s.plane;
+    const double f = a.fin[p + si + off], g = fma(om, scaled(sum, E - 1023 + e - kCoefH) - f, f);
+    a.fout[p + si] = g;
+    for (int k = 0; k < nimg; ++k) a.fout[p + img[k]] = g;
+  };
+#pragma unroll 1
+  for (int g = 0; g < T::ND; ++g)
+#pragma unroll 1
+    for (int r = tb.dir_first[g]; r < tb.dir_first[g + 1]; ++r)
+#pragma unroll 1
+      for (int m = 0; m < 8; ++m)
+        relax(tb.first8[r] + m, tb.off8[r][m], tb.H8[r], tb.dir_n[g], 7, m, tb.er8[r] + tb.rho8[r]);
+#pragma unroll 1
+  for (int r = 0; r < T::NT; ++r) {
+    const int mask = tail_mask<ORDER>(r);
+#pragma unroll 1
+    for (int m = 0; m < T::LT; ++m)
+      relax(tb.firstT[r] + m, tb.offT[r][m], tb.HT[r], tb.nT[r], mask, spread(mask, m), tb.erT[r] + tb.rhoT[r]);
+  }
+}
+
 template <int ORDER>
 __global__ void __launch_bounds__(128, ORDER == 2 ? 6 : 5) k_step3x(const __grid_constant__ Tables3x<ORDER> tb,
                                                                     const __grid_constant__ Step3Args<double> a) {
@@ -317,7 +359,6 @@ __global__ void __launch_bounds__(128, ORDER == 2 ? 6 : 5) k_step3x(const __grid
   const Column R{M.s + K * 128};                              // the rates of a direction pattern
   int uf, ue, eo;            // see below
   long long O0, W[3];        // tau^-1 U0 and tau^-1 U^i / |n|, in units of 2^(eo - 62)
-  bool ok;
   {
     long long m[kMom3];
     int E;
@@ -325,7 +366,7 @@ __global__ void __launch_bounds__(128, ORDER == 2 ? 6 : 5) k_step3x(const __grid
     double N[4], T00, t[3], S[6];
     moment_values(m, tb.sk, N, T00, t, S);
     const Cell3 c = landau3x(N, T00, t, S);
-    ok = c.ok && E > 128 && E < 2040;
+    const bool ok = c.ok && E > 128 && E < 2040;
     const double U[3] = {c.u[0] * c.U0, c.u[1] * c.U0, c.u[2] * c.U0};
     double Mk[K];
     mj_moments3x<K>(c, U, Mk);
@@ -333,9 +374,22 @@ __global__ void __launch_bounds__(128, ORDER == 2 ? 6 : 5) k_step3x(const __grid
     float sum = 0.f;
 #pragma unroll
     for (int k = 0; k < K; ++k) sum += fabsf(cut_float(Mk[k])) * __uint_as_float((unsigned)(127 + tb.hk[k]) << 23);
-    const double o0 = s.inv_tau * c.U0;
+    const double o0 = s.inv_tau * c.U0, kl = s.inv_tau * tb.inv_len;
     const int xg = above(sum), xo = above(2.f * cut_float(o0));
-    ok = ok && xg < 60 && xg > -60;
+    // (moments within the float range, and, as in step2x.cu, rates below 64)
+    const bool fits = between(c.n, -28, 28) && between(c.L, -28, 28) && between(c.U0, -1, 10) && between(o0, -1000, 6);
+    if (__builtin_expect(!(ok && fits && xg < 60 && xg > -60), 0)) {
+      // no Landau frame: counted, left unrelaxed (a population that is not finite becomes NaN)
+      if (!ok) atomicAdd(a.status, 1ULL);
+      double* const v = (double*)M.s;
+#pragma unroll
+      for (int k = 0; k < K; ++k) v[k * 128] = ok ? Mk[k] : 0.0;
+      v[K * 128] = ok ? o0 : 0.0;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) v[(K + 1 + i) * 128] = ok ? kl * U[i] : 0.0;
+      relax_plain3<ORDER>(tb, a, v, ok ? E : 1023, x, y, z);
+      return;
+    }
     // the unit 2^(u - kBits) of a run: u = max(its populations' exponent + uf, rho + ue)
     uf = max(0, xo - 2);
     ue = E + xg + max(0, xo - 3);
@@ -343,7 +397,6 @@ __global__ void __launch_bounds__(128, ORDER == 2 ? 6 : 5) k_step3x(const __grid
     for (int k = 0; k < K; ++k) M.set(k, scaled_integer(Mk[k], tb.hk[k] + 62 - xg));
     eo = max(xo, -2);
     O0 = scaled_integer(o0, 62 - eo);
-    const double kl = s.inv_tau * tb.inv_len;
 #pragma unroll
     for (int i = 0; i < 3; ++i) W[i] = scaled_integer(kl * U[i], 62 - eo);
   }
@@ -353,23 +406,6 @@ __global__ void __launch_bounds__(128, ORDER == 2 ? 6 : 5) k_step3x(const __grid
     long long wide[26];
     nimg = cell_images(s, x, y, z, wide);
     for (int i = 0; i < nimg; ++i) img[i] = (int)(wide[i] - si);
-  }
-  if (!ok) {
-    // no Landau frame: counted, left unrelaxed (a population that is not finite becomes NaN)
-    atomicAdd(a.status, 1ULL);
-#pragma unroll 1
-    for (int r = 0; r < T::N8 + T::NT; ++r) {
-      const int first = r < T::N8 ? tb.first8[r] : tb.firstT[r - T::N8];
-      const int* off = r < T::N8 ? tb.off8[r] : tb.offT[r - T::N8];
-#pragma unroll 1
-      for (int m = 0; m < (r < T::N8 ? 8 : T::LT); ++m) {
-        const long long p = (long long)(first + m) * P;
-        const double f = base[p + off[m]], g = fma(0.0, -f, f);
-        ob[p] = g;
-        for (int i = 0; i < nimg; ++i) ob[p + img[i]] = g;
-      }
-    }
-    return;
   }
   const long long half = 1LL << (29 - eo);                  // half a unit of the relaxation's sum
   const int sE = ue - max(0, uf - 1);                       // E + xg

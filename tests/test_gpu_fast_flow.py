@@ -67,7 +67,7 @@ def _draws(H, f):
 
 
 @pytest.mark.parametrize("order", [2, 3])
-@pytest.mark.parametrize("u", [0.9, 0.95, 0.99, 0.995, 0.999])
+@pytest.mark.parametrize("u", [0.9, 0.95, 0.99, 0.995, 0.999, 0.9999])
 def test_step3_of_a_uniform_stream(rl, order, u):
     """A uniform equilibrium stream: a step of its stored populations against the
     oracle's.  The bar is the oracle's amplification of rounding errors of the

@@ -98,3 +98,50 @@ def test_relaxation_time_fields_of_any_value(rl, m, order, stream):
         assert (np.abs(got - want).max(0)[ok] <= bar[ok]).all()
         lat.set_populations(start)
     lat.close()
+
+
+@pytest.mark.parametrize("order", [2, 3, 4, 5])
+@pytest.mark.parametrize("wall", [2.0, 1e4, 1e8, 1e12])
+def test_walls_of_any_temperature(rl, order, wall):
+    """(1+1)-d: the equilibrium of a wall cell is a polynomial of the prescribed
+    temperature, whose terms are all positive or as large as f itself at T >> 1: each
+    wall cell to 1e-13 of its largest value, as its few roundings make."""
+    from oracle import d1 as O1
+    nx = 40
+    one = np.ones(nx)
+    lat = rl.Lattice1(nx, order=order, tau=0.9, boundary="eqwall_x", wall_T=(wall, 0.5 * wall), precision="fp64")
+    q = O1.massless_quadrature_1d(order)
+    sim = O1.Simulation1(q, nx, tau=0.9, boundary="eqwall_x", wall_T=(wall, 0.5 * wall))
+    for s in (lat, sim):
+        s.init(one, 0 * one, one)
+        s.step(1)
+    assert lat.sync_status() == (0, 0)
+    pos = {(int(d), round(float(p), 9)): i for i, (d, p) in enumerate(zip(lat.n, lat.p[:, 0]))}
+    got = lat.populations()[[pos[(int(d), round(float(p), 9))] for d, p in zip(q.n, q.p[:, 0])]]
+    for x in (0, nx - 1):
+        assert rel_linf(got[:, x], sim.fs[:, x]) <= 1e-13 * (1 if order < 5 else 10)
+    assert rel_linf(got[:, 1:-1], sim.fs[:, 1:-1]) <= 1e-12
+    lat.close()
+
+
+@pytest.mark.parametrize("order,u", [(2, 0.9), (2, 0.999), (2, 0.9999), (2, 0.99999), (3, 0.9), (3, 0.999), (3, 0.9999),
+                                     (5, 0.9), (5, 0.999)])
+def test_fast_streams_in_one_dimension(rl, order, u):
+    """A uniform stream (rates from e^theta / tau, 400 at the last speed): a step of
+    its stored populations against the oracle's, at 16 times the oracle's own
+    amplification of roundings sum_k |H_ik M_k| 2^-53 (as in test_gpu_fast_flow.py)."""
+    from oracle import d1 as O1
+    from tests.test_gpu_fast_flow import _draws
+    one = np.ones(37)
+    lat = rl.Lattice1(37, order=order, tau=0.8, precision="fp64")
+    q = O1.massless_quadrature_1d(order)
+    pos = {(int(d), round(float(p), 9)): i for i, (d, p) in enumerate(zip(lat.n, lat.p[:, 0]))}
+    idx = [pos[(int(d), round(float(p), 9))] for d, p in zip(q.n, q.p[:, 0])]
+    lat.init(one, u * one, one)
+    draws = _draws(rl.plan1(order)["H"], lat.populations()[:, 0])[idx]
+    fs, fields = O1.collide1(draws, q, O1.Expansion1(q), 0.8)
+    assert fields.ok.all()
+    lat.step(1)
+    assert lat.sync_status() == (0, 0)
+    assert rel_linf(lat.populations()[idx], fs[:, :1]) <= 16 * 2.0 ** (40 - 53) * rel_linf(fs[:, 1:], fs[:, :1])
+    lat.close()
