@@ -131,3 +131,28 @@ def test_step2_of_a_uniform_stream(rl, m, order, u):
     assert lat.sync_status() == (0, 0)
     assert rel_linf(lat.populations()[idx], fs[:, :1]) <= bar
     lat.close()
+
+
+@pytest.mark.parametrize("order,speeds", [(2, (0.9, 0.95, 0.98, 0.99, 0.993, 0.995)), (3, (0.9, 0.95, 0.98, 0.99))])
+def test_fp32_step3_of_uniform_streams(rl, order, speeds):
+    """FP32 storage, 24 directions: a step of the stored populations against the
+    oracle's, the bar as for FP64 at four roundings of 2^-24 (each moment is one
+    FP32 sum over 12 or 39 runs).  A frame is found in every cell."""
+    plan = rl.plan3(order)
+    quad = OD.massless_quadrature_3d(order)
+    one = np.ones((6, 6, 6))
+    for u in speeds:
+        d = np.random.default_rng(3).standard_normal((24, 3))
+        for v in u * d / np.linalg.norm(d, axis=1)[:, None]:
+            lat = rl.Lattice3(6, 6, 6, tau=0.8, precision="fp32", order=order)
+            idx = _order3(lat, quad)
+            lat.init(one, *[c * one for c in v], one)
+            draws = _draws(plan["H"], lat.populations()[:, 0, 0, 0])[idx]
+            fs, fields = OD.collide3(draws, quad, OD.Expansion3(quad, order), 0.8)
+            assert fields.ok.all()
+            lat.step(1)
+            assert lat.sync_status() == (0, 0)
+            bar = 4 * 2.0 ** (40 - 24) * rel_linf(fs[:, 1:], fs[:, :1])
+            err = rel_linf(lat.populations()[idx], fs[:, :1, None, None])
+            assert err <= bar, (u, err, bar)
+            lat.close()
