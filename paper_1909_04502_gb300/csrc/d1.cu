@@ -258,7 +258,7 @@ __device__ __noinline__ void relax_plain1(const Tab1x<N>& tb, double* v, int E, 
   }
 }
 
-template <int N>
+template <int N, bool SLOW>
 __global__ void __launch_bounds__(kThreads) k_step1x(const __grid_constant__ Tab1x<N> tb, const __grid_constant__ Sc s,
                                                      const double* __restrict__ before, double* __restrict__ fout,
                                                      unsigned long long* status) {
@@ -285,10 +285,11 @@ __global__ void __launch_bounds__(kThreads) k_step1x(const __grid_constant__ Tab
     c.T2 = Tw > 0.0 ? 0.5 * Tw : c.T2;
     c.eth[0] = c.eth[1] = om[0] = om[1] = 1.0;
   }
-  const int xo = above(fmaxf(cut_float(om[0]), cut_float(om[1]))), eo = max(xo, -2), uf = max(0, xo - 2);
-  const long long half = 1LL << max(29 - eo, 0);
+  const int xo = above(fmaxf(cut_float(om[0]), cut_float(om[1]))), eo = max(xo, SLOW ? kSlowestRate : -2),
+            uf = max(0, xo - 2), sb = SLOW ? max(-eo, 0) : 0;
+  const long long half = 1LL << max(29 - eo - sb, 0);
   // (moments within the float range, and, as in step2x.cu, rates below 64)
-  const bool fits = between(c.n, -28, 28) && between(c.T2, -28, 12) && between(c.eth[0], -8, 8) && xo <= 6;
+  const bool fits = c.E > 320 && between(c.n, -28, 28) && between(c.T2, -28, 12) && between(c.eth[0], -8, 8) && xo <= 6;
 #pragma unroll
   for (int d = 0; d < 2; ++d) {
     double m[N];
@@ -332,9 +333,14 @@ __global__ void __launch_bounds__(kThreads) k_step1x(const __grid_constant__ Tab
       split_balanced(C - X, dh, dl);
       Acc q{0, half};
       macs(q, Cx{oh, ol}, dh, dl);
-      X += collect(q, 2 + eo);
+      const long long change = collect(q, 2 + eo + sb);
       const int k = u + tb.er[j] - kBits;
-      g[i] = __builtin_expect(hi32(X) > 0, 1) ? from_fixed_positive(X, k) : from_fixed_any(X, k);
+      if constexpr (SLOW) {
+        g[i] += from_fixed(change, k - sb);
+      } else {
+        X += change;
+        g[i] = __builtin_expect(hi32(X) > 0, 1) ? from_fixed_positive(X, k) : from_fixed_any(X, k);
+      }
     }
   }
   store_cell1<Q>(s, fout, x, g);
@@ -738,7 +744,7 @@ dim3 grid1(int nx) { return dim3((nx + kThreads - 1) / kThreads); }
 
 template <int N>
 cudaError_t launch_step1x(const Tab1x<N>& t, const rlbm1_handle* h) {
-  return rlbm::launch_chained(true, k_step1x<N>, grid1(h->sc.nx), dim3(kThreads), 0, h->stream, t, h->sc,
+  return rlbm::launch_chained(true, h->sc.tau <= rlbm::kSlowTau ? k_step1x<N, false> : k_step1x<N, true>, grid1(h->sc.nx), dim3(kThreads), 0, h->stream, t, h->sc,
                               (const double*)h->buf[h->cur], (double*)h->buf[h->cur ^ 1], h->status);
 }
 

@@ -11,12 +11,14 @@
 // Precision.  Moments: X_i = f_i 2^(e_i) in units of 2^(E - 59) or 2^(E - 60), e_i a constant
 // of the table (the exponent of p0^2, so that 2^-59 is relative to the largest
 // contribution to T^00) and 2^E above them all.  Relaxation: f and f^eq of a
-// run in units of 2^(u - 58), 2^u above the run's own populations and, with
+// run in units of 2^(u - 59), 2^u above the run's own populations and, with
 // kHead spare bits, above every |term| sum of its equilibrium rows: finer than
 // the rounding of an FP64 sum over the same terms.  Additions are exact.
-// Products with a table constant c = h 2^32 + l (60 or 62 bits, l signed, as
+// Products with a table constant c = h 2^32 + l (61 or 63 bits, l signed, as
 // the value's lower half is) keep the partial products h xh, h xl and l xh
-// exactly and drop l xl, a zero-mean 2^-60 of the full scale at most.
+// exactly and drop l xl, a zero-mean 2^-61 of the full scale at most.  With one bit
+// less in the relaxation and its constants a step of the order-3 and order-5 tables was up
+// to 3 times as far off as one in FP64.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -24,12 +26,12 @@
 
 namespace rlbm {
 
-constexpr int kBits = 58;        // populations in a relaxation: |X| < 2^kBits
+constexpr int kBits = 59;        // populations in a relaxation: |X| < 2^kBits
 constexpr int kBitsM = 59;       // populations in the moment sums: runs of 8 members
 constexpr int kBitsM4 = 60;      // ... and of at most 4
 constexpr int kHead = 4;         // results of a relaxation: below 2^(kBits + kHead)
 constexpr int kCoefM = 63;       // moment constants: their sum over the runs at most 2^kCoefM
-constexpr int kCoefH = 60;       // equilibrium constants: a row's sum over a parity class at most four
+constexpr int kCoefH = 61;       // equilibrium constants (kBits + 2): a row's sum over a parity class at most four
 
 // constant c = h 2^32 + l with l in [-2^31, 2^31)
 struct Cx {
@@ -130,7 +132,7 @@ __host__ __device__ __forceinline__ long long to_fixed_cut(double f, int d) {
   return (long long)shift_right(m << (BITS - 53), d);
 }
 
-// The double nearest to Y 2^(k - 1023), |Y| < 2^62, k + 62 < 2047 and k > 0.
+// The double nearest to Y 2^(k - 1023), |Y| < 2^63, k + 62 < 2047 and k > 0.
 __host__ __device__ __forceinline__ double from_fixed(long long Y, int k) {
   const unsigned long long A = Y < 0 ? 0ULL - (unsigned long long)Y : (unsigned long long)Y;
   const unsigned ah = (unsigned)(A >> 32);
@@ -147,7 +149,7 @@ __host__ __device__ __forceinline__ double from_fixed(long long Y, int k) {
   return double_of(w ? r : 0ULL);
 }
 
-// the same for 2^32 <= Y < 2^62
+// the same for 2^32 <= Y
 __host__ __device__ __forceinline__ double from_fixed_positive(long long Y, int k) {
 #ifdef __CUDA_ARCH__
   const int lz = __clz(hi32(Y));

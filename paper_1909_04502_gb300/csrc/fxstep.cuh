@@ -46,6 +46,15 @@ __device__ __forceinline__ int run_exponent(const double (&f)[L], bool& plain) {
   return (int)(h >> 20);
 }
 
+// Slow relaxation, tau above kSlowTau or of a field: the unit of a run stands above
+// every |term| of its equilibrium, up to 2^10 times the populations, so that a population
+// that hardly changes would lose bits to it at each step.  There (SLOW) only the
+// change, rate times difference, is taken in fixed point, in a unit finer by the
+// rate (to 2^kSlowestRate), and added to the population in FP64: one addition more
+// per population, the rounding of an FP64 step.
+constexpr double kSlowTau = 2.0;
+constexpr int kSlowestRate = -28;
+
 // Signed, subnormal and non-finite values: out of line, so that the loops of
 // the usual case stay short.
 __device__ __noinline__ long long to_fixed_any(double f, int d) { return to_fixed(f, d - biased_exponent(f)); }

@@ -322,7 +322,7 @@ __device__ __noinline__ void relax_plain2(const Tables2x& tb, const StepArgs<dou
   if (tb.nr) relax(tb.firstr, tb.Hr, 0.0, 0.0, o0, tb.err + tb.rhor);
 }
 
-template <int K, int MODE, bool MASSLESS>
+template <int K, int MODE, bool MASSLESS, bool SLOW>
 __global__ void __launch_bounds__(kThreads2x, K == 9 || MODE == kOnLattice ? 5 : 4) k_step2x(const __grid_constant__ Tables2x tb,
                                                                         const __grid_constant__ StepArgs<double> a,
                                                                         double inv_tau) {
@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(kThreads2x, K == 9 || MODE == kOnLattice ? 5 :
     else return __ldg(base + tb.off[i]);
   };
 
-  int uf, ue, eo;            // the unit 2^(u - kBits) of a quartet: u = max(its exponent + uf, rho + ue)
+  int uf, ue, eo, sb = 0;    // the unit 2^(u - kBits) of a quartet: u = max(its exponent + uf, rho + ue)
   long long O0, W[2];        // tau^-1 U0 and vscale tau^-1 U^i in units of 2^(eo - 62)
   {
     long long m[9];
@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(kThreads2x, K == 9 || MODE == kOnLattice ? 5 :
     // less than FP64 would be left of it)
     const bool rate = (__double2hiint(o0) & 0x7FFFFFFF) < (1023 + 6) << 20;      // finite, |o0| < 2^6
     // (moments within the float range, whatever U and T within these)
-    const bool fits = between(c.n, -28, 28) && between(c.L, -28, 28) && between(c.T, -30, 24) && between(c.U0, -1, 10);
+    const bool fits = E > 320 && between(c.n, -28, 28) && between(c.L, -28, 28) && between(c.T, -30, 24) && between(c.U0, -1, 10);
     if (__builtin_expect(!(ok && rate && fits && xg < 60 && xg > -60), 0)) {
       // no Landau frame: counted, left unrelaxed (a population that is not finite becomes NaN)
       if (!ok) atomicAdd(a.status, 1ULL);
@@ -405,14 +405,15 @@ __global__ void __launch_bounds__(kThreads2x, K == 9 || MODE == kOnLattice ? 5 :
       if (has_lo<K, MASSLESS>(k)) v += scaled_integer(lo[k], tb.hk[k] + 62 - xg);
       M.set(k, v);
     }
-    eo = max(xo, -2);
+    eo = max(xo, SLOW ? kSlowestRate : -2);
+    if constexpr (SLOW) sb = max(-eo, 0);
     O0 = scaled_integer(o0, 62 - eo);
     W[0] = scaled_integer(kl * Ux, 62 - eo);
     W[1] = scaled_integer(kl * Uy, 62 - eo);
   }
   const bool edge = (s.boundary == 0 ? (x < s.hx || x >= s.nx - s.hx) : (x == 0 || x == s.nx - 1)) || y < s.hy ||
                     y >= s.ny - s.hy;
-  const long long half = 1LL << (29 - eo);                  // half a unit of the relaxation's sum
+  const long long half = 1LL << (29 - eo - sb);             // half a unit of the relaxation's sum
   const int sE = ue - max(0, uf - 1);                       // E + xg
   // relaxation of a set of L populations from its class sums C (in units of 2^(rho + sE - 64 + ...)) and rates R
   auto relax = [&](auto tag, int first, int er, int rho, long long (&C)[decltype(tag)::value], auto&& transform) {
@@ -444,10 +445,13 @@ __global__ void __launch_bounds__(kThreads2x, K == 9 || MODE == kOnLattice ? 5 :
       const int2 om = R.get(m);
       Acc q{0, half};
       macs(q, Cx{om.x, om.y}, dh, dl);
-      X[m] += collect(q, 2 + eo);
+      const long long change = collect(q, 2 + eo + sb);
+      if constexpr (SLOW) f[m] += from_fixed(change, k - sb);
+      X[m] += change;
       low = min(low, hi32(X[m]));
     }
-    if (__builtin_expect(low > 0, 1)) {
+    if constexpr (SLOW) {
+    } else if (__builtin_expect(low > 0, 1)) {
 #pragma unroll
       for (int m = 0; m < L; ++m) f[m] = from_fixed_positive(X[m], k);
     } else {
@@ -569,21 +573,23 @@ cudaError_t launch_fields(const Tables2x& tb, const MomentArgs<double>& a, cudaS
   return cudaGetLastError();
 }
 
-template <int K, int MODE, bool MASSLESS>
+template <int K, int MODE, bool MASSLESS, bool SLOW>
 cudaError_t launch2x(const Tables2x& tb, const StepArgs<double>& a, cudaStream_t st) {
   const dim3 block = block2x(a.s.ny), grid = grid2x(a.s, block);
   const size_t bytes = shared2x(K, MODE, tb.Q);
+  const auto kernel = k_step2x<K, MODE, MASSLESS, SLOW>;
   if (bytes > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(k_step2x<K, MODE, MASSLESS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)shared2x(K, MODE, kMaxQ));
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shared2x(K, MODE, kMaxQ));
     if (e != cudaSuccess) return e;
   }
-  return launch_chained(!a.s.plain, k_step2x<K, MODE, MASSLESS>, grid, block, bytes, st, tb, a, 1.0 / a.s.tau);
+  return launch_chained(!a.s.plain, kernel, grid, block, bytes, st, tb, a, 1.0 / a.s.tau);
 }
 
 template <int K, int MODE>
 cudaError_t launch2x(const Tables2x& tb, const StepArgs<double>& a, cudaStream_t st) {
-  return a.s.massless ? launch2x<K, MODE, true>(tb, a, st) : launch2x<K, MODE, false>(tb, a, st);
+  if (a.s.tau_mode != 0 || !(a.s.tau <= kSlowTau))
+    return a.s.massless ? launch2x<K, MODE, true, true>(tb, a, st) : launch2x<K, MODE, false, true>(tb, a, st);
+  return a.s.massless ? launch2x<K, MODE, true, false>(tb, a, st) : launch2x<K, MODE, false, false>(tb, a, st);
 }
 
 }  // namespace

@@ -341,7 +341,7 @@ __device__ __noinline__ void relax_plain3(const Tables3x<ORDER>& tb, const Step3
   }
 }
 
-template <int ORDER>
+template <int ORDER, bool SLOW>
 __global__ void __launch_bounds__(128, ORDER == 2 ? 6 : 5) k_step3x(const __grid_constant__ Tables3x<ORDER> tb,
                                                                     const __grid_constant__ Step3Args<double> a) {
   using T = Tables3x<ORDER>;
@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(128, ORDER == 2 ? 6 : 5) k_step3x(const __grid
 
   const Column M{limbs + threadIdx.y * 32 + threadIdx.x};   // basis moments in units of 2^(xg - 62) 2^E
   const Column R{M.s + K * 128};                              // the rates of a direction pattern
-  int uf, ue, eo;            // see below
+  int uf, ue, eo, sb = 0;    // see below
   long long O0, W[3];        // tau^-1 U0 and tau^-1 U^i / |n|, in units of 2^(eo - 62)
   {
     long long m[kMom3];
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(128, ORDER == 2 ? 6 : 5) k_step3x(const __grid
     const double o0 = s.inv_tau * c.U0, kl = s.inv_tau * tb.inv_len;
     const int xg = above(sum), xo = above(2.f * cut_float(o0));
     // (moments within the float range, and, as in step2x.cu, rates below 64)
-    const bool fits = between(c.n, -28, 28) && between(c.L, -28, 28) && between(c.U0, -1, 10) && between(o0, -1000, 6);
+    const bool fits = E > 320 && between(c.n, -28, 28) && between(c.L, -28, 28) && between(c.U0, -1, 10) && between(o0, -1000, 6);
     if (__builtin_expect(!(ok && fits && xg < 60 && xg > -60), 0)) {
       // no Landau frame: counted, left unrelaxed (a population that is not finite becomes NaN)
       if (!ok) atomicAdd(a.status, 1ULL);
@@ -395,7 +395,8 @@ __global__ void __launch_bounds__(128, ORDER == 2 ? 6 : 5) k_step3x(const __grid
     ue = E + xg + max(0, xo - 3);
 #pragma unroll
     for (int k = 0; k < K; ++k) M.set(k, scaled_integer(Mk[k], tb.hk[k] + 62 - xg));
-    eo = max(xo, -2);
+    eo = max(xo, SLOW ? kSlowestRate : -2);
+    if constexpr (SLOW) sb = max(-eo, 0);
     O0 = scaled_integer(o0, 62 - eo);
 #pragma unroll
     for (int i = 0; i < 3; ++i) W[i] = scaled_integer(kl * U[i], 62 - eo);
@@ -407,7 +408,7 @@ __global__ void __launch_bounds__(128, ORDER == 2 ? 6 : 5) k_step3x(const __grid
     nimg = cell_images(s, x, y, z, wide);
     for (int i = 0; i < nimg; ++i) img[i] = (int)(wide[i] - si);
   }
-  const long long half = 1LL << (29 - eo);                  // half a unit of the relaxation's sum
+  const long long half = 1LL << (29 - eo - sb);             // half a unit of the relaxation's sum
   const int sE = ue - max(0, uf - 1);                       // E + xg
   // f^eq of a run of L members from its row, and their relaxation at the rates R
   auto relax_run = [&](auto tag, const Cx* H, const int* off, int first, int er, int rho, int mask) {
@@ -454,10 +455,13 @@ __global__ void __launch_bounds__(128, ORDER == 2 ? 6 : 5) k_step3x(const __grid
       const int2 om = R.get(m);
       Acc q{0, half};
       macs(q, Cx{om.x, om.y}, dh, dl);
-      X[m] += collect(q, 2 + eo);
+      const long long change = collect(q, 2 + eo + sb);
+      if constexpr (SLOW) f[m] += from_fixed(change, k - sb);
+      X[m] += change;
       low = min(low, hi32(X[m]));
     }
-    if (__builtin_expect(low > 0, 1)) {
+    if constexpr (SLOW) {
+    } else if (__builtin_expect(low > 0, 1)) {
 #pragma unroll
       for (int m = 0; m < L; ++m) f[m] = from_fixed_positive(X[m], k);
     } else {
@@ -538,7 +542,8 @@ dim3 grid3x(const Scalars3& s) { return dim3((s.nx + 31) / 32, (s.ny + 3) / 4, s
 template <int ORDER>
 cudaError_t launch_step3x(const Tables3x<ORDER>& tb, const Step3Args<double>& a, cudaStream_t st) {
   if (a.s.Q != Tables3x<ORDER>::Q) return cudaErrorInvalidValue;
-  k_step3x<ORDER><<<grid3x(a.s), dim3(32, 4), 0, st>>>(tb, a);
+  if (!(a.s.tau <= kSlowTau)) k_step3x<ORDER, true><<<grid3x(a.s), dim3(32, 4), 0, st>>>(tb, a);
+  else k_step3x<ORDER, false><<<grid3x(a.s), dim3(32, 4), 0, st>>>(tb, a);
   return cudaGetLastError();
 }
 template <int ORDER, typename S>
