@@ -198,6 +198,11 @@ __device__ __forceinline__ Cell1 macro1x(const Tab1x<N>& tb, const S (&g)[2 * N]
         plain = plain && (unsigned)h < 0x7FF00000U;
         e = max(e, ((h & 0x7FF00000) >> 20) + tb.ep[j]);
       }
+      if (__builtin_expect(!plain, 0)) {
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+          if ((__double2hiint(g[2 * j + s]) & 0x7FF00000) == 0x7FF00000) e = kNotFinite;
+      }
       Es[s] = e + 1;
 #pragma unroll
       for (int j = 0; j < N; ++j) {
@@ -209,7 +214,7 @@ __device__ __forceinline__ Cell1 macro1x(const Tab1x<N>& tb, const S (&g)[2 * N]
     } else {
       int e = tb.ref_E - 1;
 #pragma unroll
-      for (int j = 0; j < N; ++j) e = max(e, (int)((__float_as_uint(g[2 * j + s]) >> 23) & 0xFF) + 896 + 1 + tb.ep[j]);
+      for (int j = 0; j < N; ++j) e = max(e, float_exponent(__float_as_uint(g[2 * j + s]) & 0x7FFFFFFFU) + 1 + tb.ep[j]);
       Es[s] = e + 1;
 #pragma unroll
       for (int j = 0; j < N; ++j)
@@ -240,7 +245,7 @@ __device__ __forceinline__ Cell1 macro1x(const Tab1x<N>& tb, const S (&g)[2 * N]
   c.T2 = quotient(c.l2, c.n);
   const float fB = fminf(cut_float(c.B[0]), cut_float(c.B[1])), fn = cut_float(c.n), fT = cut_float(c.T2);
   c.ok = fB > 1e-30f && fn > 1e-30f && fn < 1e30f && fT > 1e-30f && fT < 1e30f && c.E > 128 &&
-         c.E < (sizeof(S) == 4 ? 1140 : 2040);
+         c.E < 2040;
   return c;
 }
 
@@ -347,7 +352,8 @@ __global__ void __launch_bounds__(kThreads) k_step1x(const __grid_constant__ Tab
 }
 
 // Fields of the streamed populations (pull = 1) or of the stored ones:
-// out[8][nx] = n, ux, T, eps, N0, Nx, T00, T0x (n NaN without a Landau frame).
+// out[8][nx] = n, ux, T, eps, N0, Nx, T00, T0x (n NaN without a Landau frame, all NaN
+// where a population is not finite).
 template <int N, typename S>
 __global__ void __launch_bounds__(kThreads) k_fields1x(const __grid_constant__ Tab1x<N> tb, const __grid_constant__ Sc s,
                                                        const S* __restrict__ fin, int pull, double* out) {
@@ -361,6 +367,10 @@ __global__ void __launch_bounds__(kThreads) k_fields1x(const __grid_constant__ T
   const Cell1 c = macro1x<N, S>(tb, g);
   const int nx = s.nx, k = c.E - 1023;
   const double T00 = c.B[0] + c.B[1], T0x = c.B[0] - c.B[1];
+  if (__builtin_expect(c.E > kNotFinite / 2, 0)) {
+    for (int j = 0; j < 8; ++j) out[j * nx + x] = __longlong_as_double(0x7ff8000000000000LL);
+    return;
+  }
   out[x] = c.ok ? scaled(c.n, k) : __longlong_as_double(0x7ff8000000000000LL);
   out[nx + x] = T0x * reciprocal(fma(2.0, c.l2, T00));
   out[2 * nx + x] = 2.0 * c.T2;

@@ -31,7 +31,12 @@ __device__ __forceinline__ void add_product(long long& m, Cx c, int xh, int xl) 
   m = a.H + (long long)hi32(a.M);
 }
 
-// The largest biased exponent of a run, and whether every member is finite and not negative.
+// The exponent that stands for an infinity or NaN: the scale of the sums then lies
+// above that of every finite value.
+constexpr int kNotFinite = 1 << 14;
+
+// The largest biased exponent of a run (kNotFinite: a member is not finite), and whether
+// every member is finite and not negative.
 template <int L>
 __device__ __forceinline__ int run_exponent(const double (&f)[L], bool& plain) {
   unsigned h = 0;
@@ -42,6 +47,7 @@ __device__ __forceinline__ int run_exponent(const double (&f)[L], bool& plain) {
     h = 0;
 #pragma unroll
     for (int q = 0; q < L; ++q) h = max(h, (unsigned)__double2hiint(f[q]) & 0x7FF00000U);
+    if (h == 0x7FF00000U) return kNotFinite;
   }
   return (int)(h >> 20);
 }
@@ -59,6 +65,11 @@ constexpr int kSlowestRate = -28;
 // the usual case stay short.
 __device__ __noinline__ long long to_fixed_any(double f, int d) { return to_fixed(f, d - biased_exponent(f)); }
 __device__ __noinline__ double from_fixed_any(long long Y, int k) { return from_fixed(Y, k); }
+
+// the same exponent of a float
+__device__ __forceinline__ int float_exponent(unsigned magnitude) {
+  return magnitude < 0x7F800000U ? (int)(magnitude >> 23) + 896 : kNotFinite;
+}
 
 // g 2^ep (a float, exact) in units of 2^(E - BITS): d = E - 1 - ep - 896 + 63 - BITS.
 __device__ __forceinline__ long long float_units(float g, int d) {

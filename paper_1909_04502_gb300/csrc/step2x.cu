@@ -554,16 +554,18 @@ __global__ void __launch_bounds__(kThreads2x, 8) k_fields2x(const __grid_constan
   if (!ok) atomicAdd(a.status, 1ULL);
   const int cell = y * s.nx + x;
   const int k2 = E - 1023;
+  const double nan = __longlong_as_double(0x7ff8000000000000LL);
+  const bool finite = E < kNotFinite / 2;                // (the populations)
   const double f[5] = {scaled(c.n, k2), c.u[0], c.u[1], c.T, scaled(c.L, k2)};
 #pragma unroll
   for (int k = 0; k < 5; ++k)
-    if (a.out[k]) a.out[k][cell] = f[k];
+    if (a.out[k]) a.out[k][cell] = finite ? f[k] : nan;
 #pragma unroll
   for (int j = 0; j < 3; ++j)
-    if (a.N) a.N[(size_t)j * s.ncell + cell] = scaled(v[j], k2);
+    if (a.N) a.N[(size_t)j * s.ncell + cell] = finite ? scaled(v[j], k2) : nan;
 #pragma unroll
   for (int j = 0; j < 6; ++j)
-    if (a.Tab) a.Tab[(size_t)j * s.ncell + cell] = scaled(v[3 + j], k2);
+    if (a.Tab) a.Tab[(size_t)j * s.ncell + cell] = finite ? scaled(v[3 + j], k2) : nan;
 }
 
 template <int MODE, bool MASSLESS>

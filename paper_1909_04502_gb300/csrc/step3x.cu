@@ -89,7 +89,7 @@ __device__ __forceinline__ void run_units(const float (&g)[L], int ep, long long
   unsigned h = 0;
 #pragma unroll
   for (int q = 0; q < L; ++q) h = max(h, __float_as_uint(g[q]) & 0x7FFFFFFFU);
-  raise_scale<1>(m, E, (int)(h >> 23) + 896 + ep + 1);
+  raise_scale<1>(m, E, float_exponent(h) + ep + 1);
   const int d = E - 1 - ep - 896 + 63 - kBitsM;
   const long long r = ref >> min(E - ref_E, 63);
 #pragma unroll
@@ -512,7 +512,8 @@ __global__ void __launch_bounds__(128, ORDER == 2 ? 6 : 5) k_step3x(const __grid
 }
 
 // Fields of f(t): the populations pulled from f*(t-1) (after a step) or, at
-// t = 0, f*(0) = f^eq itself: n, ux, uy, uz, T, eps (n NaN without a Landau frame).
+// t = 0, f*(0) = f^eq itself: n, ux, uy, uz, T, eps (n NaN without a Landau frame, all of
+// them NaN where a population is not finite).
 template <int ORDER, typename S>
 __global__ void __launch_bounds__(128, ORDER == 2 ? 7 : 6) k_fields3x(const __grid_constant__ Tables3x<ORDER> tb,
                                                   const __grid_constant__ Fields3Args<S> a) {
@@ -525,14 +526,16 @@ __global__ void __launch_bounds__(128, ORDER == 2 ? 7 : 6) k_fields3x(const __gr
   double N[4], T00, t[3], Sm[6];
   moment_values(m, tb.sk, N, T00, t, Sm);
   const Cell3 c = landau3x(N, T00, t, Sm);
-  const bool ok = c.ok && E > 128 && E < (sizeof(S) == 4 ? 1140 : 2040);   // (an infinity or NaN lies above)
+  const bool ok = c.ok && E > 128 && E < 2040;
+  const double nan = __longlong_as_double(0x7ff8000000000000LL);
+  const bool finite = E < kNotFinite / 2;
   const long long cell = ((long long)z * s.ny + y) * s.nx + x, nc = (long long)s.nx * s.ny * s.nz;
-  a.out[cell] = ok ? scaled(c.n, E - 1023) : __longlong_as_double(0x7ff8000000000000LL);
-  a.out[nc + cell] = c.u[0];
-  a.out[2 * nc + cell] = c.u[1];
-  a.out[3 * nc + cell] = c.u[2];
-  a.out[4 * nc + cell] = quotient(third(c.L), c.n);
-  a.out[5 * nc + cell] = scaled(c.L, E - 1023);
+  a.out[cell] = ok ? scaled(c.n, E - 1023) : nan;
+  a.out[nc + cell] = finite ? c.u[0] : nan;
+  a.out[2 * nc + cell] = finite ? c.u[1] : nan;
+  a.out[3 * nc + cell] = finite ? c.u[2] : nan;
+  a.out[4 * nc + cell] = finite ? quotient(third(c.L), c.n) : nan;
+  a.out[5 * nc + cell] = finite ? scaled(c.L, E - 1023) : nan;
 }
 
 dim3 grid3x(const Scalars3& s) { return dim3((s.nx + 31) / 32, (s.ny + 3) / 4, s.nz); }

@@ -145,3 +145,66 @@ def test_fast_streams_in_one_dimension(rl, order, u):
     assert lat.sync_status() == (0, 0)
     assert rel_linf(lat.populations()[idx], fs[:, :1]) <= 16 * 2.0 ** (40 - 53) * rel_linf(fs[:, 1:], fs[:, :1])
     lat.close()
+
+
+def _row3(precision, order, n):
+    """Fields of a line of cells at rest, T = 1, of densities n along x, at t = 0."""
+    from paper_1909_04502_gb300 import rlbm
+    shape = (6, 6, len(n))
+    lat = rlbm.Lattice3(len(n), 6, 6, tau=0.9, precision=precision, order=order)
+    one = np.ones(shape)
+    lat.init(np.ascontiguousarray(n * one), 0 * one, 0 * one, 0 * one, one)
+    mo = {k: v[2, 3] for k, v in lat.moments().items()}
+    lat.close()
+    return mo
+
+
+def _row1(precision, order, n):
+    from paper_1909_04502_gb300 import rlbm
+    lat = rlbm.Lattice1(len(n), order=order, tau=0.9, precision=precision)
+    lat.init(n, 0 * n, 1 + 0 * n)
+    mo = lat.moments()
+    lat.close()
+    return mo
+
+
+@pytest.mark.parametrize("row,order", [(_row3, 2), (_row3, 3), (_row1, 3), (_row1, 5)])
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_fields_up_to_the_largest_populations(rl, row, order, precision):
+    """Densities to the end of the storage's range have their fields, to its
+    rounding; from where a population is infinite no field is finite."""
+    top = 1e37 if precision == "fp32" else 1e300
+    n = np.array([1.0, 1e20, 1e30, 1e34, 1e35, 1e36, 5e36, top, 3.0, 1e45 if precision == "fp32" else np.inf, np.nan, 2.0])
+    tol = 1e-4 if precision == "fp32" else 1e-10
+    mo = row(precision, order, n)
+    good = np.isfinite(n) & (n <= top)
+    with np.errstate(invalid="ignore"):
+        assert np.abs(mo["n"] / n - 1)[good].max() <= tol and np.abs(mo["T"] - 1)[good].max() <= tol
+    for k in ("n", "T", "eps", "ux"):
+        assert np.isfinite(mo[k][good]).all() and not np.isfinite(mo[k][~good]).any(), k
+
+
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("m,order,steps", [(0.0, 2, 0), (0.0, 2, 1), (5.0, 3, 0), (5.0, 3, 1)])
+def test_full_moments_of_non_finite_populations(rl, m, order, steps, bad):
+    """N^a and T^ab of a cell with a population that is not finite are not finite,
+    as their sums in FP64 are; those of the cells that it has not reached are."""
+    nx, ny = 40, 30
+    lat = rl.Lattice(nx, ny, m=m, order=order, tau=0.9, precision="fp64")
+    one = np.ones((ny, nx))
+    lat.init(one, 0 * one, 0 * one, one)
+    f = lat.populations()
+    f[3, 15, 20] = bad
+    lat.set_populations(f)
+    lat.step(steps)
+    mo = lat.moments(full=True)
+    y, x = 15, 20
+    if steps:
+        x, y = x + lat.n[3][0], y + lat.n[3][1]          # where it has moved
+    far = one.astype(bool)
+    far[y, x] = False
+    for k, v in mo.items():
+        v = v.reshape(-1, ny, nx)
+        assert not np.isfinite(v[:, y, x]).any(), k
+        assert np.isfinite(v[:, far]).all(), k
+    lat.close()
