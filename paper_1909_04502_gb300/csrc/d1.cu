@@ -278,8 +278,6 @@ __global__ void __launch_bounds__(kThreads) k_step1x(const __grid_constant__ Tab
   Cell1 c = macro1x<N, double>(tb, g);
   if (!c.ok) {
     atomicAdd(status, 1ULL);                                 // left unrelaxed (Omega = 0)
-#pragma unroll
-    for (int i = 0; i < Q; ++i) g[i] = fma(0.0, -g[i], g[i]);
     store_cell1<Q>(s, fout, x, g);
     return;
   }

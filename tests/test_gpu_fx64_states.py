@@ -208,3 +208,35 @@ def test_full_moments_of_non_finite_populations(rl, m, order, steps, bad):
         assert not np.isfinite(v[:, y, x]).any(), k
         assert np.isfinite(v[:, far]).all(), k
     lat.close()
+
+
+@pytest.mark.parametrize("boundary", ["periodic", "freeflow_x", "eqwall_x"])
+@pytest.mark.parametrize("order", [2, 3, 5])
+def test_cells_without_a_frame_in_one_dimension(rl, order, boundary):
+    """(1+1)-d, FP64: cells of negative density, at both ends and inside, and one with
+    infinite (order 2) or NaN populations are counted and their populations
+    streamed as they are, infinities included."""
+    nx = 41
+    n, u, T = np.ones(nx), np.full(nx, 0.1), np.ones(nx)
+    for x in (0, 13, nx - 1):
+        n[x] = -1.0
+    n[20], u[20], T[20] = 1.7e308, 0.3, 3.0                    # n T overflows
+    lat = rl.Lattice1(nx, order=order, tau=0.9, boundary=boundary, precision="fp64")
+    lat.init(n, u, T)
+    lat.sync_status()
+    f = lat.populations()
+    assert np.isinf(f[:, 20]).any() if order == 2 else np.isnan(f[:, 20]).any()
+    s = np.ravel(lat.n)
+    src = np.arange(nx)[None] - s[:, None]
+    src = src % nx if boundary == "periodic" else np.clip(src, 0, nx - 1)
+    g = np.take_along_axis(f, src, 1)                          # streamed
+    p = lat.p[:, :1]
+    with np.errstate(invalid="ignore"):
+        B = [(p * p * g)[s == k].sum(0) for k in (1, -1)]
+        none = ~((B[0] > 0) & (B[1] > 0) & np.isfinite(g).all(0))
+    lat.step(1)
+    got = lat.populations()
+    assert lat.sync_status() == (-4, none.sum()) and none.sum() >= 4
+    assert np.array_equal(got[:, none], g[:, none], equal_nan=True)
+    assert np.isfinite(got[:, ~none]).all()
+    lat.close()
