@@ -171,7 +171,9 @@ int rlbm_step_kernel(const rlbm_handle* h);
 /* Landau-frame fields of f(t) (steps 1-4 of Sec. 6.2).  Every output is
  * nullable; n, ux, uy, T, eps: nx*ny FP64; Nab: 3*nx*ny (N^0, N^x, N^y
  * planes); Tab: 6*nx*ny (T^00, T^0x, T^0y, T^xx, T^xy, T^yy planes).
- * With on_device = 0 the call copies to host and synchronises. */
+ * With on_device = 0 the call copies to host and synchronises; with
+ * on_device = 1 the planes are device memory, of any device and alignment (those
+ * that are not 8-byte aligned memory of the current device by a copy). */
 int rlbm_moments(rlbm_handle* h, double* n, double* ux, double* uy, double* T,
                  double* eps, double* Nab, double* Tab, int on_device);
 

@@ -3,6 +3,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <cstring>
 #include <memory>
 #include <string>
@@ -201,6 +202,19 @@ bool orbit_symmetric(const rlbm_handle* h) {
 int effective_step_kernel(const rlbm_handle* h) {
   if (h->step_kernel != RLBM_KERNEL_AUTO) return h->step_kernel;
   return RLBM_KERNEL_DIRECT;
+}
+
+// Whether a kernel may store doubles at p: aligned memory of the current device.
+// (Another device's needs peer access, which a copy does not.)
+bool kernel_writable(const double* p) {
+  cudaPointerAttributes at;
+  int device;
+  if (reinterpret_cast<uintptr_t>(p) % sizeof(double)) return false;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&device) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == device);
 }
 
 template <typename R>
@@ -681,11 +695,11 @@ int rlbm_moments(rlbm_handle* h, double* n, double* ux, double* uy, double* T, d
   const Scalars& s = h->sc;
   const int mode = h->p.stream_mode == RLBM_BILINEAR ? kBilinear : kOnLattice;
   const void* fin = h->have_prev ? h->buf[h->cur ^ 1] : h->buf[h->cur];
-  // device outputs are written by the kernel itself; host outputs go through the field planes
-  double* host[7] = {n, ux, uy, T, eps, Nab, Tab};
+  // planes that the kernel can store into it writes itself, others go through the field planes
+  double* to[7] = {n, ux, uy, T, eps, Nab, Tab};
   double* dev[7];
   for (int k = 0; k < 7; ++k)
-    dev[k] = !host[k] || on_device ? host[k] : h->fields + (size_t)(k == 6 ? 8 : k) * s.ncell;
+    dev[k] = !to[k] || (on_device && kernel_writable(to[k])) ? to[k] : h->fields + (size_t)(k == 6 ? 8 : k) * s.ncell;
   auto fill = [&](auto& a) {
     for (int k = 0; k < 5; ++k) a.out[k] = dev[k];
     a.N = dev[5];
@@ -703,11 +717,13 @@ int rlbm_moments(rlbm_handle* h, double* n, double* ux, double* uy, double* T, d
     e = h->tx ? launch_fields2x(*h->tx, a, mode, h->stream) : launch_fields<double>(*h->td, a, mode, h->stream);
   }
   if (e != cudaSuccess) return cuda_fail(h, e, "fields kernel");
-  if (on_device) return RLBM_OK;
   for (int k = 0; k < 7; ++k) {
     const size_t bytes = (size_t)(k < 5 ? 1 : k == 5 ? 3 : 6) * s.ncell * sizeof(double);
-    if (host[k]) RLBM_CUDA(h, cudaMemcpyAsync(host[k], dev[k], bytes, cudaMemcpyDeviceToHost, h->stream));
+    if (to[k] != dev[k])
+      RLBM_CUDA(h, cudaMemcpyAsync(to[k], dev[k], bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                                   h->stream));
   }
+  if (on_device) return RLBM_OK;
   RLBM_CUDA(h, cudaStreamSynchronize(h->stream));
   return RLBM_OK;
 }
