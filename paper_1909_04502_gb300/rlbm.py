@@ -159,10 +159,10 @@ def make_params(nx, ny, m=0.0, order=2, quadrature=None, groups=None, v0=0.0, cu
     p.quadrature = QUAD[quadrature]
     keep = []
     if groups is not None:
-        g = np.ascontiguousarray(np.asarray(groups, dtype=np.int32).reshape(-1))
-        keep.append(g)
-        p.groups = g.ctypes.data_as(_IP)
-        p.n_groups = len(g) // 2
+        vecs = np.ascontiguousarray(np.asarray(groups, dtype=np.int32).reshape(-1))
+        keep.append(vecs)
+        p.groups = vecs.ctypes.data_as(_IP)
+        p.n_groups = len(vecs) // 2
     p.v0 = float(v0)
     if custom is not None:
         c = np.ascontiguousarray(np.asarray(custom, dtype=np.float64).reshape(-1, 6))
