@@ -103,10 +103,10 @@ __host__ __device__ inline Frame64 frame64(double E, const double (&t)[3], const
     // positive definite, so that Newton from l = E, which is never below the root, comes down to it
     l = E;
 #pragma unroll 1
-    for (int it = 0; it < 60; ++it) {
+    for (int it = 0; it < 40; ++it) {
       solve();
       const double d = energy() / w;
-      if (!(id > 0.0 && w > 0.0)) break;
+      if (!(id > 0.0 && w > 0.0 && l > 0.0)) break;
       l += d;
       if (!(fabs(d) > 1e-6 * l)) break;
     }

@@ -291,18 +291,19 @@ constexpr size_t shared2x(int K, int mode, int Q) {
 // streamed populations, or null where they are read again.
 template <int K>
 __device__ __noinline__ void relax_plain2(const Tables2x& tb, const StepArgs<double>& a, const double* v, const double* kept,
-                                          const double* base, int E, int x, int y) {
+                                          const double* base, int E, bool frame, int x, int y) {
   const Scalars& s = a.s;
   const double o0 = v[K * kThreads2x], kx = v[(K + 1) * kThreads2x], ky = v[(K + 2) * kThreads2x];
   // sx, sy: the signs of the odd members of p^x and p^y, 0 where the row has none
   auto relax = [&](int i, const Cx* H, double sx, double sy, double om, int e) {
     double sum = 0.0;
+    if (!frame) om = 0.0;
 #pragma unroll 1
-    for (int k = 0; k < K; ++k) {
+    for (int k = 0; frame && k < K; ++k) {
       sum = fma((mono_ax(k) ? sx : 1.0) * (mono_ay(k) ? sy : 1.0) * constant_value(H[k], tb.hk[k]), v[k * kThreads2x], sum);
     }
     const double f = kept ? kept[i * kThreads2x] : __ldg(base + tb.off[i]);
-    const double g = fma(om, scaled(sum, E - 1023 + e - kCoefH) - f, f);
+    const double g = fma(om, (frame ? scaled(sum, E - 1023 + e - kCoefH) : 0.0) - f, f);
     a.fout[(base - a.fin) + (long long)i * s.iplane] = g;
     for_each_halo_image(s, x, y, [&](long long hi) { a.fout[hi + (long long)i * s.iplane] = g; });
   };
@@ -389,12 +390,12 @@ __global__ void __launch_bounds__(kThreads2x, K == 9 || MODE == kOnLattice ? 5 :
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         const double f = has_lo<K, MASSLESS>(k) ? Mk[k] + lo[k] : Mk[k];
-        v[k * kThreads2x] = ok ? f : 0.0;
+        v[k * kThreads2x] = f;
       }
-      v[K * kThreads2x] = ok ? o0 : 0.0;
-      v[(K + 1) * kThreads2x] = ok ? kl * Ux : 0.0;
-      v[(K + 2) * kThreads2x] = ok ? kl * Uy : 0.0;
-      relax_plain2<K>(tb, a, v, kept2x(K, MODE) ? F : nullptr, base, ok ? E : 1023, x, y);
+      v[K * kThreads2x] = o0;
+      v[(K + 1) * kThreads2x] = kl * Ux;
+      v[(K + 2) * kThreads2x] = kl * Uy;
+      relax_plain2<K>(tb, a, v, kept2x(K, MODE) ? F : nullptr, base, E, ok, x, y);
       return;
     }
     uf = max(0, xo - 2);

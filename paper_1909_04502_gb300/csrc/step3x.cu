@@ -305,7 +305,7 @@ __device__ __forceinline__ void mj_moments3x(const Cell3& c, const double (&U)[3
 // column of the shared memory).
 template <int ORDER>
 __device__ __noinline__ void relax_plain3(const Tables3x<ORDER>& tb, const Step3Args<double>& a, const double* v, int E,
-                                          int x, int y, int z) {
+                                          bool frame, int x, int y, int z) {
   using T = Tables3x<ORDER>;
   const Scalars3& s = a.s;
   const long long si = sidx3(s, x, y, z);
@@ -313,15 +313,19 @@ __device__ __noinline__ void relax_plain3(const Tables3x<ORDER>& tb, const Step3
   const int nimg = cell_images(s, x, y, z, img);
   // the member of a run that negates the components of neg
   auto relax = [&](int i, int off, const Cx* H, const int* n, int mask, int neg, int e) {
-    double sum = 0.0, om = v[T::K * 128];
+    double sum = 0.0, om = 0.0;
+    if (frame) {
 #pragma unroll 1
-    for (int k = 0; k < T::K; ++k)
-      if (!(kPar3[k] & ~mask))
-        sum = fma((__popc(kPar3[k] & neg) & 1) ? -v[k * 128] : v[k * 128], constant_value(H[k], tb.hk[k]), sum);
-    for (int c = 0; c < 3; ++c)
-      if (mask >> c & 1) om = fma((neg >> c & 1) ? (double)n[c] : -(double)n[c], v[(T::K + 1 + c) * 128], om);
+      for (int k = 0; k < T::K; ++k)
+        if (!(kPar3[k] & ~mask))
+          sum = fma((__popc(kPar3[k] & neg) & 1) ? -v[k * 128] : v[k * 128], constant_value(H[k], tb.hk[k]), sum);
+      sum = scaled(sum, E - 1023 + e - kCoefH);
+      om = v[T::K * 128];
+      for (int c = 0; c < 3; ++c)
+        if (mask >> c & 1) om = fma((neg >> c & 1) ? (double)n[c] : -(double)n[c], v[(T::K + 1 + c) * 128], om);
+    }
     const long long p = (long long)i * s.plane;
-    const double f = a.fin[p + si + off], g = fma(om, scaled(sum, E - 1023 + e - kCoefH) - f, f);
+    const double f = a.fin[p + si + off], g = fma(om, sum - f, f);
     a.fout[p + si] = g;
     for (int k = 0; k < nimg; ++k) a.fout[p + img[k]] = g;
   };
@@ -383,11 +387,11 @@ __global__ void __launch_bounds__(128, ORDER == 2 ? 6 : 5) k_step3x(const __grid
       if (!ok) atomicAdd(a.status, 1ULL);
       double* const v = (double*)M.s;
 #pragma unroll
-      for (int k = 0; k < K; ++k) v[k * 128] = ok ? Mk[k] : 0.0;
-      v[K * 128] = ok ? o0 : 0.0;
+      for (int k = 0; k < K; ++k) v[k * 128] = Mk[k];
+      v[K * 128] = o0;
 #pragma unroll
-      for (int i = 0; i < 3; ++i) v[(K + 1 + i) * 128] = ok ? kl * U[i] : 0.0;
-      relax_plain3<ORDER>(tb, a, v, ok ? E : 1023, x, y, z);
+      for (int i = 0; i < 3; ++i) v[(K + 1 + i) * 128] = kl * U[i];
+      relax_plain3<ORDER>(tb, a, v, E, ok, x, y, z);
       return;
     }
     // the unit 2^(u - kBits) of a run: u = max(its populations' exponent + uf, rho + ue)

@@ -240,3 +240,70 @@ def test_cells_without_a_frame_in_one_dimension(rl, order, boundary):
     assert np.array_equal(got[:, none], g[:, none], equal_nan=True)
     assert np.isfinite(got[:, ~none]).all()
     lat.close()
+
+
+@pytest.mark.parametrize("m,order,stream", [(0.0, 2, "onlattice"), (0.0, 3, "onlattice"), (5.0, 3, "onlattice"),
+                                            (10.0, 2, "onlattice"), (0.0, 2, "bilinear"), (0.0, 3, "bilinear")])
+def test_flows_without_frames_only_stream(rl, m, order, stream):
+    """Negative densities everywhere, on the faces too: each step only streams (on the
+    lattice bit by bit, bilinear to its four roundings), through the images that the
+    steps themselves have stored."""
+    nx, ny, steps = 37, 7, 3
+    lam = 0.9 if stream == "bilinear" else 0.0
+    y, x = np.meshgrid(np.arange(ny), np.arange(nx), indexing="ij")
+    lat = rl.Lattice(nx, ny, m=m, order=order, tau=0.9, precision="fp64", stream=stream, lam=lam)
+    lat.init(-1 - 0.1 * np.cos(x + y), 0.1 * np.cos(1.0 * y), 0.1 + 0.0 * x, 1 + 0.1 * np.sin(1.0 * x))
+    lat.sync_status(raise_on_error=False)
+    f = lat.populations()
+    lat.step(steps)
+    assert lat.sync_status(raise_on_error=False) == (-4, steps * nx * ny)
+    for _ in range(steps):
+        f = OS.stream_onlattice(f, lat.n) if lam == 0 else OS.stream_bilinear(f, lam * lat.p[:, 1:] / lat.p[:, :1], "periodic")
+    if lam == 0:
+        assert np.array_equal(lat.populations(), f)
+    else:
+        assert np.abs(lat.populations() - f).max() <= steps * 4 * 2.0 ** -53 * np.abs(f).max()
+    lat.close()
+
+
+@pytest.mark.parametrize("precision,order", [("fp64", 2), ("fp64", 3), ("fp32", 2), ("fp32", 3)])
+def test_flows_without_frames_only_stream_in_three_dimensions(rl, precision, order):
+    from oracle import d3 as OD
+    nx, ny, nz, steps = 35, 7, 6, 3
+    z, y, x = np.meshgrid(np.arange(nz), np.arange(ny), np.arange(nx), indexing="ij")
+    lat = rl.Lattice3(nx, ny, nz, tau=0.9, precision=precision, order=order)
+    lat.init(-3 - 0.1 * np.cos(x + y + z), 0.1 * np.cos(1.0 * y), 0.1 + 0.0 * x, 0.1 * np.sin(1.0 * z), 1 + 0.1 * np.sin(1.0 * x))
+    lat.sync_status()
+    f = lat.populations()
+    lat.step(steps)
+    assert lat.sync_status() == (-4, steps * nx * ny * nz)
+    for _ in range(steps):
+        f = OD.stream3(f, lat.n)
+    assert np.array_equal(lat.populations(), f)
+    lat.close()
+
+
+@pytest.mark.parametrize("order", [2, 3])
+def test_infinite_populations_in_three_dimensions(rl, order):
+    """A corner cell of infinite density: the populations that are not finite arrive as
+    NaN, each in a cell that is counted and keeps its others; the rest is finite."""
+    nx, ny, nz = 35, 13, 14
+    one = np.ones((nz, ny, nx))
+    n = one.copy()
+    n[0, 0, 0] = np.inf
+    lat = rl.Lattice3(nx, ny, nz, tau=0.9, precision="fp64", order=order)
+    lat.init(n, 0.1 * one, 0 * one, 0 * one, one)
+    lat.sync_status()
+    f = lat.populations()
+    hit = np.zeros((nz, ny, nx), bool)
+    for i in np.flatnonzero(~np.isfinite(f[:, 0, 0, 0])):
+        hit[tuple(lat.n[i][::-1] % (nz, ny, nx))] = True
+    assert hit.sum() > 10
+    lat.step(1)
+    got = lat.populations()
+    assert lat.sync_status() == (-4, hit.sum())
+    for i, s in enumerate(lat.n):
+        g = np.roll(f[i], (int(s[2]), int(s[1]), int(s[0])), (0, 1, 2))
+        assert np.array_equal(got[i][hit], np.where(np.isfinite(g), g, np.nan)[hit], equal_nan=True)
+    assert np.isfinite(got[:, ~hit]).all()
+    lat.close()
