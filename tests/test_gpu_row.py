@@ -63,3 +63,54 @@ def test_row_equals_equal_rows(rl, nx, kw, steps):
             assert np.abs(g[:, r] - w[:, hy]).max() <= tol
     for lat in lats:
         lat.close()
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(stream="bilinear", lam=1.0), dict(m=1.0, boundary="eqwall_x", g=(1e-5, 2e-5))])
+@pytest.mark.parametrize("steps", [1024, 1025, 2048, 2051])
+def test_long_calls_equal_short_ones(rl, kw, steps):
+    """A call is split into launches of at most 1024 steps: both buffers, images
+    included, are bit by bit those of calls of at most 100."""
+    nx = 150
+    rng = np.random.default_rng(5)
+    row = [1 + 0.2 * rng.random((1, nx)), 0.2 * rng.random((1, nx)), 0.1 * rng.random((1, nx)), 1 + 0.1 * rng.random((1, nx))]
+    out = []
+    for size in (steps, 100):
+        lat = rl.Lattice(nx, 1, precision="fp32", tau=0.8, **kw)
+        lat.init(*row)
+        for done in range(0, steps, size):
+            lat.step(min(size, steps - done))
+        assert lat.sync_status() == (0, 0) and lat.t == steps
+        out.append(_storage(lat)[0])
+        lat.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("shape", [0, 1, 2])
+def test_rows_in_a_batch_and_by_the_direct_kernel(rl, shape):
+    """One-row members of a batch (whose chains launch the row's kernel unchained) and the
+    direct kernel: the same bits, and the batch's rows go on by themselves."""
+    cfg = [dict(nx=150, ny=1, tau=0.8), dict(nx=33, ny=1, tau=1.1, m=1.0), dict(nx=2049, ny=1, tau=0.7, m=10.0),
+           dict(nx=40, ny=24, tau=0.9), dict(nx=70, ny=1, tau=0.8, stream="bilinear", lam=1.0)]
+    batch = rl.Batch([dict(c, precision="fp32") for c in cfg])
+    lats = []
+    for i, c in enumerate(cfg):
+        rng = np.random.default_rng(i)
+        s = (c["ny"], c["nx"])
+        f = [1 + 0.2 * rng.random(s), 0.2 * rng.random(s), 0.1 * rng.random(s), 1 + 0.1 * rng.random(s)]
+        lat = rl.Lattice(precision="fp32", **c)
+        lat.set_step_kernel("direct")
+        for x in (lat, batch[i]):
+            x.init(*f)
+        lats.append(lat)
+    batch.config(shape, batch.info()["grid_max"][shape] if shape < 2 else 0)
+    for k in (7, 4):
+        batch.step(k)
+        batch[0].step(3)
+        for lat in lats:
+            lat.step(k)
+        lats[0].step(3)
+        assert batch.sync_status() == (0, 0)
+        for i, lat in enumerate(lats):
+            assert np.array_equal(batch[i].populations(), lat.populations()), i
+    batch.close()
