@@ -354,6 +354,17 @@ int rlbm_adjoint_step(rlbm_handle* h, const void* x_prev, const void* a_next, vo
 int rlbm_convert_f32_f64(const float* in_f, double* out_d, int nf, const double* in_d, float* out_f, int nd,
                          void* stream);
 
+/* The short arithmetic of the fixed-point FP64 steps and of the (3+1)-d FP32
+ * frame, element by element on device arrays of n (asynchronous on `stream`).
+ * rlbm_fast_math_f64: out has 6 planes of n: 1 / b, a / b, 1 / sqrt(b) (b > 0,
+ * within an ulp of the exact value), a cut to FP32, a rounded to FP32 for
+ * finite values, and 1 where that conversion reports a value that no float
+ * holds.  rlbm_fast_math_f32: 3 planes: a / b in FP32 (b normal, below 2^126),
+ * a widened to FP64 (zero becomes 2^-127), and a widened for finite values.
+ * No counterpart in the paper: a check of the library's own arithmetic. */
+int rlbm_fast_math_f64(const double* a, const double* b, double* out, int n, void* stream);
+int rlbm_fast_math_f32(const float* a, const float* b, double* out, int n, void* stream);
+
 /* Message of the last error on this handle (or of the last failed
  * rlbm_create when h is NULL).  Never NULL. */
 const char* rlbm_last_error(const rlbm_handle* h);

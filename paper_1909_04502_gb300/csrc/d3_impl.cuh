@@ -1,6 +1,6 @@
 // Device helpers of the (3+1)-d massless steps (step3.cu: order 2; step3q.cu:
-// order 3): layout, periodic images, the 4 x 4 Landau frame (Sec. 4) in FP64
-// and in FP32 with an FP64 correction, and the Maxwell-Juttner moments of the
+// order 3; step3x.cu: FP64): layout, periodic images, the 4 x 4 Landau frame
+// (Sec. 4) in FP32 with an FP64 correction, and the Maxwell-Juttner moments of the
 // bases kBasis3 / kBasis3o3 (App. B, d = 3, m = 0).
 #pragma once
 #include <cuda_runtime.h>
@@ -364,12 +364,12 @@ __device__ __forceinline__ void moments_run8(const S (&F)[8], const C* c, S (&m)
   m[13] = fma((S)c[13], F[0], m[13]);
 }
 
-// The periodic images of a cell next to a face, copied from the
+// FP32 storage: the periodic images of a cell next to a face, copied from the
 // values the thread has just stored for the cell itself, B populations at a
 // time so that B loads are in flight (one at a time, each waits on the L2
 // round trip of the one before, as the stores in between may alias them).
-template <int QT, int B, typename S>
-__device__ __forceinline__ void images_from_stored(const Scalars3& s, S* out, long long si, int x, int y, int z) {
+template <int QT, int B>
+__device__ __forceinline__ void images_from_stored(const Scalars3& s, float* out, long long si, int x, int y, int z) {
   int ix[2], iy[2], iz[2];
   const int nx2 = images1(x, s.nx, s.h, ix), ny2 = images1(y, s.ny, s.h, iy), nz2 = images1(z, s.nz, s.h, iz);
   if (nx2 + ny2 + nz2 == 0) return;
@@ -384,12 +384,12 @@ __device__ __forceinline__ void images_from_stored(const Scalars3& s, S* out, lo
   static_assert(QT % B == 0, "whole batches");
   const long long P = s.plane;
   for (int i0 = 0; i0 < QT; i0 += B) {
-    S v[B];
+    float v[B];
 #pragma unroll
     for (int j = 0; j < B; ++j) v[j] = out[(long long)(i0 + j) * P + si];
 #pragma unroll
     for (int j = 0; j < B; ++j) {
-      S* oi = out + (long long)(i0 + j) * P;
+      float* oi = out + (long long)(i0 + j) * P;
       for (int m = 0; m < nimg; ++m) oi[img[m]] = v[j];
     }
   }

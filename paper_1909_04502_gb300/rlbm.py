@@ -113,6 +113,8 @@ SIGNATURES = {
     "rlbm_adjoint_backward": (ctypes.c_int, [_VP, _VP, _VP, ctypes.c_int, _VP, _VP, _VP, _VP, ctypes.c_int]),
     "rlbm_adjoint_last_error": (ctypes.c_char_p, [_VP]),
     "rlbm_convert_f32_f64": (ctypes.c_int, [_VP, _VP, ctypes.c_int, _VP, _VP, ctypes.c_int, _VP]),
+    "rlbm_fast_math_f64": (ctypes.c_int, [_VP, _VP, _VP, ctypes.c_int, _VP]),
+    "rlbm_fast_math_f32": (ctypes.c_int, [_VP, _VP, _VP, ctypes.c_int, _VP]),
     "rlbm_last_error": (ctypes.c_char_p, [_H]),
     "rlbm_strerror": (ctypes.c_char_p, [ctypes.c_int]),
 }
