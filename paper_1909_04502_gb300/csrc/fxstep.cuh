@@ -35,9 +35,9 @@ __device__ __forceinline__ void add_product(long long& m, Cx c, int xh, int xl) 
 // above that of every finite value.
 constexpr int kNotFinite = 1 << 14;
 
-// The largest biased exponent of a run (kNotFinite: a member is not finite), and whether
-// every member is finite and not negative.
-template <int L>
+// The largest biased exponent of a run (with CHECK kNotFinite if a member is not
+// finite), and whether every member is finite and not negative.
+template <bool CHECK, int L>
 __device__ __forceinline__ int run_exponent(const double (&f)[L], bool& plain) {
   unsigned h = 0;
 #pragma unroll
@@ -47,7 +47,7 @@ __device__ __forceinline__ int run_exponent(const double (&f)[L], bool& plain) {
     h = 0;
 #pragma unroll
     for (int q = 0; q < L; ++q) h = max(h, (unsigned)__double2hiint(f[q]) & 0x7FF00000U);
-    if (h == 0x7FF00000U) return kNotFinite;
+    if (CHECK && h == 0x7FF00000U) return kNotFinite;
   }
   return (int)(h >> 20);
 }

@@ -217,7 +217,7 @@ __device__ __forceinline__ void moment_sums2x(const Tables2x& tb, F&& pull, long
   auto units = [&](auto& f, int ep, auto& X) {
     constexpr int L = sizeof(X) / sizeof(X[0]);
     bool plain;
-    raise_scale<0>(m, E, run_exponent(f, plain) + ep + 1);
+    raise_scale<0>(m, E, run_exponent<true>(f, plain) + ep + 1);
     const int d = E - 1 - ep;
     if (__builtin_expect(plain, 1)) {
 #pragma unroll
@@ -423,7 +423,7 @@ __global__ void __launch_bounds__(kThreads2x, K == 9 || MODE == kOnLattice ? 5 :
 #pragma unroll
     for (int q = 0; q < L; ++q) f[q] = again(first + q);
     bool plain;
-    const int u = max(run_exponent(f, plain) + 1 - er + uf, rho + ue);
+    const int u = max(run_exponent<false>(f, plain) + 1 - er + uf, rho + ue);
     const int j = min(u - rho - sE, 62);                    // >= 0
     const long long hj = (1LL << j) >> 1;
 #pragma unroll

@@ -71,7 +71,7 @@ template <int L>
 __device__ __forceinline__ void run_units(const double (&f)[L], int ep, long long, long long (&m)[kMom3], int& E,
                                           long long (&X)[L]) {
   bool plain;
-  raise_scale<1>(m, E, run_exponent(f, plain) + ep + 1);
+  raise_scale<1>(m, E, run_exponent<true>(f, plain) + ep + 1);
   const int d = E - 1 - ep;
   if (__builtin_expect(plain, 1)) {
 #pragma unroll
@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(128, ORDER == 2 ? 6 : 5) k_step3x(const __grid
       C[c] = h.H + (long long)hi32(h.M);
     }
     bool plain;
-    const int u = max(run_exponent(f, plain) + 1 - er + uf, rho + ue);
+    const int u = max(run_exponent<false>(f, plain) + 1 - er + uf, rho + ue);
     const int j = min(u - rho - sE, 62);                    // >= 0
     const long long hj = (1LL << j) >> 1;
 #pragma unroll
