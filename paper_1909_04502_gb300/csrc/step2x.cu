@@ -12,11 +12,14 @@
 // stencils, whose 45 to 65 doubles per thread would leave three blocks per SM:
 // they are pulled again.
 //
-// What bounds it: integer issue at 20 warps per SM (about 180 instructions per
-// population and step; the sums in FP64 held that pipe at 85 % and took 540 to
-// 980 operations per cell of it, 80 to 160 are left).  517 x 333, massless order 2:
-// 56 us per step (chained) and 18 us for the fields against 190 and 139 us; 512 x 512,
-// m = 5, order 3 (49 populations): 160 and 40 us against 445 and 300 us.
+// What bounds it: latency at 20 warps per SM.  170 (order 2) and 190 (order 3)
+// instructions per population and step fill 49 % and 39 % of the issue slots, the FP64
+// pipe is busy 50 % and 48 % (the sums in FP64 held it at 85 % and took 540 to 980
+// operations per cell of it, 80 to 160 are left); a warp waits for the arithmetic before it
+// (2.2 and 2.7 cycles per issued instruction), for shared memory and the FP64 pipe (2.0
+// and 2.7) and for the populations (1.5).  517 x 333, massless order 2: 56 us per
+// step (chained) and 18 us for the fields against 190 and 139 us; 512 x 512, m = 5,
+// order 3 (49 populations): 167 and 40 us against 445 and 300 us.
 #include <cuda_runtime.h>
 
 #include "fxstep.cuh"
@@ -75,16 +78,17 @@ __device__ __forceinline__ Cell2 landau2x(const double (&v)[9], float k, double 
     c.L += wide_double(d);
     c.u[0] += wide_double(cx);
     c.u[1] += wide_double(cy);
-    settled = fabsf(d) <= 1e-12f * l && fabsf(cx) + fabsf(cy) <= 1e-11f * w;
+    settled = fabsf(d) <= 1e-12f * l && fabsf(cx) + fabsf(cy) <= 1e-9f * w * w;
     if (it >= 1 && settled) break;
   }
   bool good = true;
   if (__builtin_expect(!(settled && det > 0.f && w > 0.f), 0)) {
-    double q[10] = {v[3], v[4], v[5], 0.0, v[6], v[7], 0.0, v[8], 0.0, 0.0};
-    good = settle_frame(q);
-    c.L = q[0];
-    c.u[0] = q[1];
-    c.u[1] = q[2];
+    const double t[3] = {v[4], v[5], 0.0}, S[6] = {v[6], v[7], 0.0, v[8], 0.0, 0.0};
+    const Frame64 f = frame64(v[3], t, S);
+    good = f.ok;
+    c.L = f.l;
+    c.u[0] = f.u[0];
+    c.u[1] = f.u[1];
   }
   const double w2 = fma(-c.u[1], c.u[1], fma(-c.u[0], c.u[0], 1.0));
   c.U0 = reciprocal_sqrt(w2);

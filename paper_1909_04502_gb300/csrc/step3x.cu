@@ -12,16 +12,18 @@
 // (App. B, d = 3, m = 0) of the cell, pass 2 pulls the populations again,
 // relaxes and stores.
 //
-// What bounds it: integer issue, about 90 instructions per population and step
-// in pass 2 and 45 in pass 1, at 40 % of the issue slots (latency of the two
-// population reads at 20 to 24 warps per SM); the FP64 pipe, which the sums
-// used to hold at 85 %, is busy 25 % with the 110 to 130 operations per cell
-// that are left.  The basis moments and the rates lie in shared-memory columns
+// What bounds it: latency at 24 (order 2) and 20 (order 3) warps per SM.  147 and 192
+// instructions per population and step fill 49 % and 41 % of the issue slots; a warp
+// waits most for the two population reads (3.4 and 3.9 cycles per issued
+// instruction), then at order 2 for the instruction cache (2.0) and in either for the
+// arithmetic before it (1.5 to 1.7).  The FP64 pipe, which the sums used to hold at 85 %,
+// is busy 31 % and 10 %, DRAM 43 % and 35 % (96^3 and 48^3).  The basis moments and the rates lie in shared-memory columns
 // so that 80 (order 2) and 96 (order 3) registers suffice; with all of them in
 // registers (128, four blocks per SM) the order-2 step ran 1.3x longer.  Signed
 // and non-finite populations leave the loop for functions of their own: inline
-// they cost the instruction cache 1.3x.  101 x 75 x 66, order 2: 0.37 ms per step
-// and 0.12 ms for the fields against 1.6 and 1.8 ms with the sums in FP64;
+// they cost the instruction cache 1.3x; the FP64 relaxation of cells
+// outside the range is out of line as well.  101 x 75 x 66, order 2: 0.38 ms per step
+// and 0.13 ms for the fields against 1.6 and 1.8 ms with the sums in FP64;
 // 192 x 192 x 6, order 3: 0.77 and 0.14 ms against 2.0 and 2.6 ms; the fields of
 // 192^3 cells in FP32 storage: 1.2 ms against 24 ms (FP64, row by row).
 #include <cuda_runtime.h>
@@ -107,7 +109,8 @@ struct Cell3 {
 // g(l) = T00 - t.(S + l)^-1 t - l, g' = u.u - 1; then (l, u) together by
 // iterative refinement: FP64 residuals of both equations, the correction
 // through the FP32 inverse.  A pass gains about 20 bits in slow flows; two are enough
-// (more run where the last still moved l by 2^-40 or u by 2^-36 of 1 - u.u).  The inverse's error
+// (more run where the last still moved l by 2^-40, or u by 2^-30 of (1 - u.u)^2: a pass
+// leaves about 2^-20 / (1 - u.u)^2 of its step).  The inverse's error
 // grows as gamma^4: what has not settled after six passes is solved in FP64
 // (frame64.cuh; from gamma of about 7 on).
 __device__ __forceinline__ Cell3 landau3x(const double (&N)[4], double T00, const double (&t)[3],
@@ -163,17 +166,17 @@ __device__ __forceinline__ Cell3 landau3x(const double (&N)[4], double T00, cons
     c.u[0] += wide_double(cx);
     c.u[1] += wide_double(cy);
     c.u[2] += wide_double(cz);
-    settled = fabsf(d) <= 1e-12f * l && fabsf(cx) + fabsf(cy) + fabsf(cz) <= 1e-11f * w;
+    settled = fabsf(d) <= 1e-12f * l && fabsf(cx) + fabsf(cy) + fabsf(cz) <= 1e-9f * w * w;
     if (it >= 1 && settled) break;
   }
   bool good = true;
   if (__builtin_expect(!(settled && det > 0.f && w > 0.f), 0)) {
-    double q[10] = {T00, t[0], t[1], t[2], S[0], S[1], S[2], S[3], S[4], S[5]};
-    good = settle_frame(q);
-    c.L = q[0];
-    c.u[0] = q[1];
-    c.u[1] = q[2];
-    c.u[2] = q[3];
+    const Frame64 f = frame64(T00, t, S);
+    good = f.ok;
+    c.L = f.l;
+    c.u[0] = f.u[0];
+    c.u[1] = f.u[1];
+    c.u[2] = f.u[2];
   }
   const double w2 = fma(-c.u[2], c.u[2], fma(-c.u[1], c.u[1], fma(-c.u[0], c.u[0], 1.0)));
   c.U0 = reciprocal_sqrt(w2);
