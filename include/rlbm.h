@@ -151,7 +151,10 @@ void rlbm_destroy(rlbm_handle* h);
 int rlbm_init(rlbm_handle* h, const double* n, const double* ux, const double* uy,
               const double* T, int on_device);
 
-/* Set the per-cell relaxation time (tau_mode RLBM_TAU_FIELD), nx*ny FP64. */
+/* Set the per-cell relaxation time (tau_mode RLBM_TAU_FIELD), nx*ny FP64.  The
+ * values are not checked: with FP64 storage a cell whose 1 / tau is not finite
+ * becomes infinite or NaN at the next step, and is counted (rlbm_sync_status)
+ * from the one after. */
 int rlbm_set_tau_field(rlbm_handle* h, const double* tau, int on_device);
 
 /* Advance nsteps time steps (asynchronous on the handle's stream). */
@@ -160,8 +163,11 @@ int rlbm_step(rlbm_handle* h, int nsteps);
 /* Choose the step kernel (RLBM_KERNEL_*); the TMA-staged kernels need FP32
  * storage, the massless Q = 28 order-2 stencil and padded rows of at least
  * 36 elements (RLBM_ERR_UNSUPPORTED otherwise).  AUTO (the default) is
- * DIRECT, the faster kernel at every grid size measured on GB300.  The kernels evaluate the same
- * expressions in the same order, so their results are bitwise identical.
+ * DIRECT, the faster kernel at every grid size measured on GB300, but for
+ * FP32 grids of one row (ny = 1) at order 2, whose steps share a kernel
+ * (rlbm_step_kernel reports DIRECT for it; choosing DIRECT launches a step at
+ * a time).  The kernels evaluate the same expressions in the same order, so
+ * their results are bitwise identical.
  * No counterpart in the paper. */
 int rlbm_set_step_kernel(rlbm_handle* h, int kernel);
 /* The kernel rlbm_step launches for this handle (RLBM_KERNEL_DIRECT,
