@@ -251,11 +251,13 @@ __device__ __forceinline__ Cell1 macro1x(const Tab1x<N>& tb, const S (&g)[2 * N]
 
 // The relaxation of one direction in FP64, for the cells whose rate or equilibrium
 // the fixed point does not hold.  v: the N populations (replaced), then the moments n T2^(a-1)
-// e^(+-a theta) in units of 2^E.  Out of line, in memory.
+// e^(+-a theta) in units of 2^E.  Behind an unlikely branch, in memory.
 template <int N>
-__device__ __noinline__ void relax_plain1(const Tab1x<N>& tb, double* v, int E, double om) {
+__device__ __forceinline__ void relax_plain1(const Tab1x<N>& tb, double* v, int E, double om) {
+#pragma unroll 1
   for (int j = 0; j < N; ++j) {
     double sum = 0.0;
+#pragma unroll 1
     for (int a = 0; a < N; ++a)
       sum = fma(rlbm::constant_value(tb.H[j][a], tb.hk[a]), v[N + a], sum);
     const double feq = rlbm::scaled(sum, E - 1023 + tb.er[j] + tb.rho[j] - rlbm::kCoefH);
